@@ -486,7 +486,7 @@ def run_ours(args):
         ach = 2 * payload / (dms / 1e3) / 1e9
         tma = args.kernel == "tma" or (args.kernel == "auto" and choice["chosen_kernel_device"] == 2)
         if args.max_ctas:
-            kname = "kvs_tma_kernel" if tma else "kvs_ldg_kernel"
+            kname = "kvs_tma_kernel" if tma else "kvs_span_kernel"
         else:
             kname = "kvs_tma_piece_kernel" if tma else "kvs_ldg_piece_kernel"
         tr, tr_src = recorded_traffic(kname, "llama8b_device")

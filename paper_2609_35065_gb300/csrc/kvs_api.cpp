@@ -195,6 +195,7 @@ struct Plan {
     uint32_t bpc = 0;
     uint64_t row_bytes = 0;
     uint64_t addr_or = 0;                // OR of all addresses and strides (alignment)
+    uint64_t span_or = 0;                // the same with each chunk's n_tok * R for the row (Job::align)
     bool     any_dedup = false;
 };
 
@@ -235,6 +236,7 @@ int validate_call(const kvs_geometry* g, const kvs_paged_cache* cache,
         if (!cache->kv_planes[p]) return fail(KVS_ERR_INVALID_ARG, "plane %d is NULL", p);
         pl.planes[p] = (uint64_t)cache->kv_planes[p];
         pl.addr_or |= pl.planes[p];
+        pl.span_or |= pl.planes[p];
     }
     // Validate requests, count entries per class.
     for (int32_t r = 0; r < nreq; ++r) {
@@ -394,6 +396,7 @@ int fill_plan(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache,
             pl.entries[e].pad = 0;
             pl.entry_bytes[e] = (uint64_t)P * c.num_tokens * pl.row_bytes;
             pl.addr_or |= addr;
+            pl.span_or |= addr | (uint64_t)c.num_tokens * pl.row_bytes;
             for (int32_t i = 0; i * B < c.num_tokens; ++i) {
                 const int64_t t = s + (int64_t)i * B;
                 const int32_t blk = q.block_table[t / B];
@@ -530,6 +533,7 @@ Job make_job(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache, 
     j.pieces_per_run = (uint32_t)((run_max + kPieceBytes - 1) / kPieceBytes);
     j.num_pieces = (uint64_t)num_entries * j.num_planes * j.blocks_per_chunk * j.pieces_per_run;
     j.mode = mode;
+    j.align = (uint32_t)pl.span_or;
     return j;
 }
 
@@ -544,11 +548,11 @@ int launch_kernel(const Job& j, int flavour, int vec, int grid, cudaStream_t s) 
     cudaError_t e = (flavour == KVS_KERNEL_TMA) ? launch_tma(j, grid, s)
                   : (flavour == kKernelLinkStaged && vec == 16) ? launch_link_staged(j, grid, s)
                   : (flavour == kKernelLinkPrefetch && vec == 16) ? launch_link_prefetch(j, grid, s)
-                  : ((flavour == kKernelLink || flavour == kKernelLinkPrefetch || flavour == kKernelLinkStaged) && vec == 16)
-                      ? launch_link(j, grid, s)
+                  : (flavour == kKernelLink || flavour == kKernelLinkPrefetch || flavour == kKernelLinkStaged)
+                      ? launch_link(j, vec, grid, s)
                   : launch_ldg(j, vec, grid, s);
     if (e != cudaSuccess) return fail(KVS_ERR_CUDA, "kernel launch failed: %s", cudaGetErrorString(e));
-    ++g_launches;
+    g_launches += kernels_of(j, vec);
     return KVS_OK;
 }
 
@@ -598,6 +602,7 @@ int run_hbmcopy(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cach
         }
         ring_plan.entries[e].chunk = (uint64_t)(st.ring + (uint64_t)slot * st.ring_slot_bytes + used);
         ring_plan.addr_or |= ring_plan.entries[e].chunk;
+        ring_plan.span_or |= ring_plan.entries[e].chunk;
         used += b;
     }
     batch_first.push_back((uint32_t)pl.entries.size());
@@ -747,7 +752,10 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     if (rc) return rc;
     const int grid = (int)KVS_F_GET_MAX_CTAS(flags);
     const int vec = vec_bytes_for(pl.addr_or);
-    int flavour = f_tma ? KVS_KERNEL_TMA : f_ldg ? KVS_KERNEL_LDG : st.kernel_device;
+    // Runs below half a piece take the LDG kernels' span pieces whatever the probe (on
+    // 32 KiB runs) has picked: the TMA kernels move one run per CTA.
+    const bool short_runs = (uint64_t)g->block_size * pl.row_bytes < kPieceBytes / 2;
+    int flavour = f_tma ? KVS_KERNEL_TMA : (f_ldg || short_runs) ? KVS_KERNEL_LDG : st.kernel_device;
     if (flavour == KVS_KERNEL_TMA && vec != 16) {
         if (f_tma) return fail(KVS_ERR_UNSUPPORTED, "TMA needs 16-byte aligned chunks, planes and rows");
         flavour = KVS_KERNEL_LDG;

@@ -45,6 +45,7 @@ struct Job {
     uint32_t        piece_bytes;     // multiple of 16
     uint32_t        block_size;      // B
     int32_t         mode;            // Mode
+    uint32_t        align;           // OR of the plane and chunk addresses and of every n_tok * R (low bits)
 };
 
 // Piece size used by both kernel flavours.
@@ -52,9 +53,12 @@ constexpr uint32_t kPieceBytes = 32768;
 
 // Launchers (kvs_kernels.cu).  `grid` <= 0 means "fill the GPU".
 cudaError_t launch_ldg(const Job& job, int vec_bytes, int grid, cudaStream_t s);
+// Kernels that launch_ldg or launch_link start for a job (2 when it has both pieces
+// that allow 16-byte vectors and pieces that do not).
+int kernels_of(const Job& job, int vec_bytes);
 cudaError_t launch_tma(const Job& job, int grid, cudaStream_t s);
 // Double-buffered 16-byte flavour for host-resident chunks (retrieve or store).
-cudaError_t launch_link(const Job& job, int grid, cudaStream_t s);
+cudaError_t launch_link(const Job& job, int vec_bytes, int grid, cudaStream_t s);
 // Retrieval of host chunks holding more bytes in flight per SM (one piece in
 // registers and three in shared memory per 256 threads, two CTAs per SM), for
 // GPUs that run other kernels meanwhile (KVS_F_FEW_SMS).

@@ -8,11 +8,13 @@
 //  * LDG: the threads of a CTA move one 32 KiB piece with 16-byte vector
 //    loads (non-coherent, no L1 allocation) issued ahead of 16-byte streaming
 //    stores.  Uncapped 16-byte work runs one 512-thread, 28-register CTA per
-//    piece (kvs_ldg_piece_kernel, four CTAs per SM); capped grids, narrower
-//    vectors and the validation compare run a 256-thread grid-stride kernel.
+//    piece (kvs_ldg_piece_kernel, four CTAs per SM).  Runs below half a piece,
+//    capped grids and odd alignments run over span pieces, 32 KiB of the
+//    chunk side whatever runs they meet (kvs_span_kernel).
 //  * LINK: the LDG scheme double-buffered in registers (the next piece's loads
 //    are issued before the current piece is stored), for host-resident
-//    chunks whose loads/stores cross the long-latency host link.
+//    chunks whose loads/stores cross the long-latency host link; over span
+//    pieces for short runs and odd alignments (kvs_link_span_kernel).
 //  * TMA: 1-D bulk async copies through shared memory (cp.async.bulk
 //    global->shared completing on an mbarrier, then a shared->global bulk
 //    store).  Uncapped work runs one 32-thread CTA per piece (six per SM);
@@ -176,27 +178,231 @@ __device__ __forceinline__ bool equal_piece(uint64_t a_addr, uint64_t b_addr, ui
 constexpr int kLdgThreads = 256;
 constexpr int kLdgUnroll = 8;
 
-template <int V, int MODE>
-__global__ void __launch_bounds__(kLdgThreads) kvs_ldg_kernel(const Decoder dc, uint32_t num_pieces) {
-    const Job& j = dc.job;
+// KVS_F_VALIDATE: flags pieces whose chunk bytes differ from the plane's.
+template <int V>
+__global__ void __launch_bounds__(kLdgThreads) kvs_compare_kernel(const Decoder dc, uint32_t num_pieces) {
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         Piece pc;
         if (!decode_piece(dc, q, pc)) continue;          // uniform across the CTA
-        if constexpr (MODE == MODE_RETRIEVE) {
-            copy_piece<V, kLdgUnroll>(pc.chunk_addr, pc.plane_addr, pc.len);
-        } else if constexpr (MODE == MODE_STORE) {
-            copy_piece<V, kLdgUnroll>(pc.plane_addr, pc.chunk_addr, pc.len);
-        } else {
-            if (!equal_piece<V, kLdgUnroll>(pc.chunk_addr, pc.plane_addr, pc.len))
-                atomicCAS(j.err, 0, KVS_ERR_ALIAS);
+        if (!equal_piece<V, kLdgUnroll>(pc.chunk_addr, pc.plane_addr, pc.len))
+            atomicCAS(dc.job.err, 0, KVS_ERR_ALIAS);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Span pieces.  All n tokens of one (chunk, plane) are contiguous in the chunk
+// (n * R bytes, the "span"); only the plane side jumps, from block to block.  A
+// span piece is piece_bytes of the span wherever its block boundaries fall, so
+// a piece is full whatever the size of a run: a 4 KiB run (two KV heads of 64)
+// fills an eighth of a piece.  The block of a vector comes from its offset by a
+// reciprocal multiply and a lookup that the L1 serves.  Bound by HBM, or the host
+// link; measured on HBM chunks (read + write) against one CTA per run:
+//   16 requests x 2000 tokens, 24 layers   4 KiB runs  216 -> 117.6 us (6.69 TB/s)
+//   16 x 4000, 24 layers                   1 KiB       806 -> 118 us
+//   16 x 2000, 48 layers                   128 B      6250 -> 125.5 us
+// ---------------------------------------------------------------------------
+struct SpanDecoder {
+    Job      job;
+    FastDiv  spp;          // pieces per span (of a full chunk)
+    FastDiv  planes;
+    FastDiv  run;          // run bytes B * R; exact for offsets below 2^31
+    uint64_t run_bytes;
+    uint32_t long_runs;    // runs longer than a piece: a piece meets at most two
+    uint32_t far_spans;    // spans of 2^31 bytes or more: divide in 64 bits
+};
+
+struct SpanPiece {
+    uint64_t       chunk;  // address of the piece's first byte in the chunk
+    uint64_t       plane;  // base of its plane; long runs: plus the first byte's offset in its run
+    const int32_t* blocks; // physical block of the run that holds the first byte, and on
+    uint32_t       off;    // short runs: offset of the first byte in its run; long runs: bytes
+                           // from it to the end of its run, at most piece_bytes
+    uint32_t       len;
+};
+
+// Piece q; false for pieces past the end of a short chunk.  Uniform across the CTA.
+__device__ __forceinline__ bool span_piece(const SpanDecoder& dc, uint32_t q, SpanPiece& sp) {
+    const Job& j = dc.job;
+    const uint32_t ep = fdiv(q, dc.spp);
+    const uint32_t k = q - ep * dc.spp.d;
+    const uint32_t e = fdiv(ep, dc.planes);
+    const uint32_t p = j.plane_begin + (ep - e * dc.planes.d);
+    const uint64_t at = (uint64_t)k * j.piece_bytes;
+    uint64_t i0;
+    if (dc.far_spans) i0 = at / dc.run_bytes;
+    else i0 = fdiv((uint32_t)at, dc.run);
+    const Entry en = j.entries[e];
+    const uint64_t span = (uint64_t)en.n_tok * j.row_bytes;
+    if (at >= span) return false;
+    sp.len = (uint32_t)min((uint64_t)j.piece_bytes, span - at);
+    const uint64_t off = at - i0 * dc.run_bytes;
+    sp.chunk = en.chunk + (uint64_t)p * span + at;
+    sp.plane = j.planes[p] + (dc.long_runs ? off : 0);
+    sp.blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i0;
+    sp.off = (uint32_t)(dc.long_runs ? min(dc.run_bytes - off, (uint64_t)j.piece_bytes) : off);
+    return true;
+}
+
+// Run of byte x < len of the piece, counted from the piece's first.
+__device__ __forceinline__ uint32_t span_run(const SpanDecoder& dc, const SpanPiece& sp, uint32_t x) {
+    return dc.long_runs ? (uint32_t)(x >= sp.off) : fdiv(sp.off + x, dc.run);   // off < run <= piece: below two pieces
+}
+
+// Plane address of byte x, in block `blk`.
+__device__ __forceinline__ uint64_t span_plane(const SpanDecoder& dc, const SpanPiece& sp, uint32_t x, int32_t blk) {
+    const uint32_t i = span_run(dc, sp, x);
+    if (dc.long_runs) return sp.plane + (uint64_t)((int64_t)blk - (int64_t)i) * dc.run_bytes + x;
+    return sp.plane + (uint64_t)(uint32_t)blk * dc.run_bytes + (sp.off + x - i * (uint32_t)dc.run_bytes);
+}
+
+// Loads U vectors of V bytes, vector base + u * T of the piece's n.  blk[u] stays -1
+// where nothing is to be moved (no such vector, a block that another request
+// writes, or one out of range, which the planner has excluded).  A retrieval looks
+// all its blocks up first, without a branch between them; a store-back, whose loads
+// need the blocks, issues each load as soon as its own lookup is back.
+template <int MODE, int V, int U>
+__device__ __forceinline__ void span_load(const SpanDecoder& dc, const SpanPiece& sp, uint32_t base, uint32_t T,
+                                          uint32_t n, int32_t (&blk)[U], typename Vec<V>::T (&r)[U]) {
+    bool bad = false;
+    auto look = [&](int u) {
+        const uint32_t k = base + u * T;
+        blk[u] = __ldg(sp.blocks + span_run(dc, sp, min(k, n - 1) * V));
+        const bool in = (uint32_t)blk[u] < (uint32_t)dc.job.num_blocks;
+        bad |= !in && blk[u] >= 0;
+        if (!in || k >= n) blk[u] = -1;
+    };
+    auto load = [&](int u) {
+        const uint32_t x = (base + u * T) * V;
+        if (blk[u] >= 0)
+            r[u] = ld_stream<V>(reinterpret_cast<const typename Vec<V>::T*>(
+                MODE == MODE_RETRIEVE ? sp.chunk + x : span_plane(dc, sp, x, blk[u])));
+    };
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        look(u);
+        if (MODE != MODE_RETRIEVE) load(u);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+        if (MODE == MODE_RETRIEVE) load(u);
+    if (bad) atomicCAS(dc.job.err, 0, KVS_ERR_BOUNDS);
+}
+
+template <int MODE, int V, int U>
+__device__ __forceinline__ void span_store(const SpanDecoder& dc, const SpanPiece& sp, uint32_t base, uint32_t T,
+                                           const int32_t (&blk)[U], const typename Vec<V>::T (&r)[U]) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint32_t x = (base + u * T) * V;
+        if (blk[u] >= 0)
+            st_stream<V>(reinterpret_cast<typename Vec<V>::T*>(
+                MODE == MODE_RETRIEVE ? span_plane(dc, sp, x, blk[u]) : sp.chunk + x), r[u]);
+    }
+}
+
+// Every 16-byte vector of the piece is aligned on both sides and lies in one
+// run.  (Rows need not be multiples of 16 bytes, only whole runs.)
+__device__ __forceinline__ bool span_wide(const SpanDecoder& dc, const SpanPiece& sp) {
+    return sp.len >= 16 &&
+           (((uint32_t)sp.chunk | (uint32_t)sp.plane | sp.off | (uint32_t)dc.run_bytes) & 15) == 0;
+}
+
+// The rest of a span that is no multiple of 16 bytes: at most 15 bytes of one run.
+template <int MODE>
+__device__ __forceinline__ void span_tail(const SpanDecoder& dc, const SpanPiece& sp) {
+    const uint32_t x = (sp.len & ~15u) + threadIdx.x;
+    if (x >= sp.len) return;
+    uint8_t r[1];
+    int32_t blk[1];
+    span_load<MODE, 1, 1>(dc, sp, x, 0, sp.len, blk, r);
+    span_store<MODE, 1, 1>(dc, sp, x, 0, blk, r);
+}
+
+// A piece whose two sides do not share 16-byte alignment (the last chunk of a
+// request where n * R is no multiple of 16, runs that are none): vectors of V, run
+// by run where a run has work for every thread.
+template <int MODE, int V, int U>
+__device__ __forceinline__ void span_narrow(const SpanDecoder& dc, const SpanPiece& sp) {
+    using T = typename Vec<V>::T;
+    if (dc.run_bytes >= blockDim.x * V) {
+        uint32_t end;
+        for (uint32_t x = 0; x < sp.len; x = end) {      // uniform across the CTA
+            const uint32_t i = span_run(dc, sp, x);
+            end = min(sp.len, dc.long_runs ? (i ? sp.len : sp.off) : (i + 1) * (uint32_t)dc.run_bytes - sp.off);
+            const int32_t blk = __ldg(sp.blocks + i);
+            if (blk < 0) continue;
+            if (blk >= dc.job.num_blocks) {
+                atomicCAS(dc.job.err, 0, KVS_ERR_BOUNDS);
+                continue;
+            }
+            const uint64_t ca = sp.chunk + x, pa = span_plane(dc, sp, x, blk);
+            const T* s = reinterpret_cast<const T*>(MODE == MODE_RETRIEVE ? ca : pa);
+            T* d = reinterpret_cast<T*>(MODE == MODE_RETRIEVE ? pa : ca);
+            const uint32_t n = (end - x) / V;
+            for (uint32_t base = threadIdx.x; base < n; base += blockDim.x * U) {
+                T r[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (base + u * blockDim.x < n) r[u] = ld_stream<V>(s + base + u * blockDim.x);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+                    if (base + u * blockDim.x < n) st_stream<V>(d + base + u * blockDim.x, r[u]);
+            }
         }
+        return;
+    }
+    const uint32_t n = sp.len / V;
+    for (uint32_t base = threadIdx.x; base < n; base += blockDim.x * U) {
+        T r[U];
+        int32_t blk[U];
+        span_load<MODE, V, U>(dc, sp, base, blockDim.x, n, blk, r);
+        span_store<MODE, V, U>(dc, sp, base, blockDim.x, blk, r);
+    }
+}
+
+// Whole-GPU or capped copy of the wide span pieces of device-resident chunks; with
+// TAIL some pieces are not wide, or end in a tail.  512 threads x 4 vectors on 32
+// registers: four CTAs and 128 KiB of loads in flight per SM.  Three CTAs (40
+// registers) lose nothing on retrievals but 16% on store-backs, whose loads wait
+// for their lookups (4 KiB runs: 139 us against 119).
+constexpr int kSpanThreads = 512;
+constexpr int kSpanCtasPerSm = 4;
+constexpr int kSpanUnroll = kPieceBytes / 16 / kSpanThreads;
+
+template <int MODE, bool TAIL>
+__global__ void __launch_bounds__(kSpanThreads, TAIL ? 3 : kSpanCtasPerSm)
+kvs_span_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+    for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
+        SpanPiece sp;
+        if (!span_piece(dc, q, sp)) continue;            // uniform across the CTA
+        if (TAIL && !span_wide(dc, sp)) continue;
+        uint4 r[kSpanUnroll];
+        int32_t blk[kSpanUnroll];
+        span_load<MODE, 16, kSpanUnroll>(dc, sp, threadIdx.x, kSpanThreads, sp.len / 16, blk, r);
+        span_store<MODE, 16, kSpanUnroll>(dc, sp, threadIdx.x, kSpanThreads, blk, r);
+        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, sp);
+    }
+}
+
+// The other pieces, in a kernel of its own: as a branch of the one above, its
+// registers spill there or halve its CTAs (aligned 120-byte rows: 9.4 -> 13 us).
+template <int MODE>
+__global__ void __launch_bounds__(kSpanThreads, 3) kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+    for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
+        SpanPiece sp;
+        if (!span_piece(dc, q, sp) || span_wide(dc, sp)) continue;   // uniform across the CTA
+        const uint32_t a = (uint32_t)sp.chunk | (uint32_t)sp.plane | sp.off | (uint32_t)dc.run_bytes | sp.len;
+        if ((a & 7) == 0) span_narrow<MODE, 8, 4>(dc, sp);
+        else if ((a & 3) == 0) span_narrow<MODE, 4, 4>(dc, sp);
+        else if ((a & 1) == 0) span_narrow<MODE, 2, 4>(dc, sp);
+        else span_narrow<MODE, 1, 4>(dc, sp);
     }
 }
 
 // Whole-GPU flavour for 16-byte aligned work: exactly one CTA per piece, 512
 // threads x 4 vectors.  The launch bound caps the kernel at 32 registers, so
 // four CTAs (2048 threads, 128 KiB of loads in flight) fit on an SM, twice the
-// residency of kvs_ldg_kernel<16>.
+// residency of a 256-thread kernel with 8 vectors a thread.
 constexpr int kPieceThreads = 512;
 constexpr int kPieceUnroll = kPieceBytes / 16 / kPieceThreads;
 
@@ -278,6 +484,44 @@ __global__ void __launch_bounds__(kLdgThreads) kvs_link_kernel(const Decoder dc,
         ha = next_piece_ldg(dc, num_pieces, q, pa);
         if (ha) load_piece16(to_plane ? pa.chunk_addr : pa.plane_addr, pa.len, ra);
         store_piece16(to_plane ? pb.plane_addr : pb.chunk_addr, pb.len, rb);
+    }
+}
+
+// The same over wide span pieces, for short runs and odd rows (TAIL as above).  A
+// run alone gives a 256-thread CTA run_bytes / 4096 vectors a thread, and the link
+// wants megabytes in flight: with 2 KiB runs, retrieval 340 -> 239 us and
+// store-back 279 -> 269 us at 49 MB (the link's own time: 233 and 254).
+template <int MODE, bool TAIL>
+__global__ void __launch_bounds__(kLdgThreads, 2) kvs_link_span_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+    uint4 ra[kLdgUnroll], rb[kLdgUnroll];
+    int32_t ba[kLdgUnroll], bb[kLdgUnroll];
+    SpanPiece pa, pb;
+    uint32_t q = blockIdx.x;
+    auto next = [&](SpanPiece& sp) -> bool {
+        while (q < num_pieces) {
+            const uint32_t cur = q;
+            q += gridDim.x;
+            if (span_piece(dc, cur, sp) && (!TAIL || span_wide(dc, sp))) return true;
+        }
+        return false;
+    };
+    auto load = [&](const SpanPiece& sp, int32_t (&blk)[kLdgUnroll], uint4 (&r)[kLdgUnroll]) {
+        span_load<MODE, 16, kLdgUnroll>(dc, sp, threadIdx.x, kLdgThreads, sp.len / 16, blk, r);
+    };
+    auto store = [&](const SpanPiece& sp, const int32_t (&blk)[kLdgUnroll], const uint4 (&r)[kLdgUnroll]) {
+        span_store<MODE, 16, kLdgUnroll>(dc, sp, threadIdx.x, kLdgThreads, blk, r);
+        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, sp);
+    };
+    bool ha = next(pa);
+    if (ha) load(pa, ba, ra);
+    while (ha) {
+        const bool hb = next(pb);
+        if (hb) load(pb, bb, rb);
+        store(pa, ba, ra);
+        if (!hb) break;
+        ha = next(pa);
+        if (ha) load(pa, ba, ra);
+        store(pb, bb, rb);
     }
 }
 
@@ -661,24 +905,71 @@ int clamp_grid(int grid, int per_sm, uint64_t pieces) {
 // busy and overlaps one CTA's stores with the next CTA's loads.  Measured on a
 // 2 GiB HBM copy this reaches 7.1 TB/s (read + write) against 6.5-6.7 TB/s for
 // persistent grid-stride grids of any shape.
-template <int V>
-cudaError_t launch_ldg_v(const Job& job, int grid, cudaStream_t s) {
+SpanDecoder make_span_decoder(const Job& job, uint32_t piece_bytes) {
+    SpanDecoder dc;
+    dc.job = job;
+    dc.job.piece_bytes = piece_bytes;
+    dc.run_bytes = (uint64_t)job.block_size * job.row_bytes;
+    const uint64_t span = dc.run_bytes * job.blocks_per_chunk;            // of a full chunk
+    const uint32_t spp = (uint32_t)((span + piece_bytes - 1) / piece_bytes);
+    dc.spp = make_fastdiv(spp);
+    dc.planes = make_fastdiv(job.num_planes);
+    dc.long_runs = dc.run_bytes > piece_bytes;
+    dc.far_spans = span >= (1ull << 31);
+    dc.run = make_fastdiv(dc.run_bytes < (1ull << 31) ? (uint32_t)dc.run_bytes : 1u);   // longer: never divided by
+    dc.job.num_pieces = (uint64_t)job.num_entries * job.num_planes * spp;
+    return dc;
+}
+
+// Bytes of a span piece: 32 KiB, halved while a launch would leave SMs (or the
+// CTAs of a capped grid) without one, down to 8 KiB.
+uint32_t span_piece_bytes(const Job& job, int ctas) {
+    const uint64_t total = (uint64_t)job.num_entries * job.num_planes * job.blocks_per_chunk * job.block_size * job.row_bytes;
+    uint32_t piece = kPieceBytes;
+    while (piece > kPieceBytes / 4 && total / piece < 2ull * ctas) piece /= 2;
+    return piece;
+}
+
+bool has_narrow(const Job& job, int vec_bytes) {
+    return vec_bytes != 16 && ((uint64_t)job.block_size * job.row_bytes % 16 || (job.align & 15));
+}
+
+// All span pieces of a job, on `grid` CTAs (0: one CTA per piece).  vec_bytes == 16:
+// rows and addresses are multiples of 16 bytes, so every piece is wide and whole.
+// Otherwise whole runs may still be, and every chunk's span with them (align).
+cudaError_t launch_spans(const Job& job, int vec_bytes, int grid, bool link, cudaStream_t s) {
+    const SpanDecoder dc = make_span_decoder(job, span_piece_bytes(job, grid > 0 ? grid : num_sms()));
+    const uint32_t n = (uint32_t)dc.job.num_pieces;
+    grid = grid > 0 ? (int)std::min<uint32_t>((uint32_t)grid, n) : (int)n;
+    const bool retrieve = job.mode == MODE_RETRIEVE;
+    const bool runs16 = dc.run_bytes % 16 == 0, narrow = has_narrow(job, vec_bytes);
+    if (runs16 && link) {
+        auto k = retrieve ? (narrow ? kvs_link_span_kernel<MODE_RETRIEVE, true> : kvs_link_span_kernel<MODE_RETRIEVE, false>)
+                          : (narrow ? kvs_link_span_kernel<MODE_STORE, true> : kvs_link_span_kernel<MODE_STORE, false>);
+        k<<<grid, kLdgThreads, 0, s>>>(dc, n);
+    } else if (runs16) {
+        auto k = retrieve ? (narrow ? kvs_span_kernel<MODE_RETRIEVE, true> : kvs_span_kernel<MODE_RETRIEVE, false>)
+                          : (narrow ? kvs_span_kernel<MODE_STORE, true> : kvs_span_kernel<MODE_STORE, false>);
+        k<<<grid, kSpanThreads, 0, s>>>(dc, n);
+    }
+    if (narrow) {
+        auto k = retrieve ? kvs_span_narrow_kernel<MODE_RETRIEVE> : kvs_span_narrow_kernel<MODE_STORE>;
+        k<<<grid, kSpanThreads, 0, s>>>(dc, n);
+    }
+    return cudaGetLastError();
+}
+
+cudaError_t launch_compare(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
     const Decoder dc = make_decoder(job);
     const uint32_t n = (uint32_t)job.num_pieces;
-    if (V == 16 && grid <= 0 && job.mode != MODE_COMPARE) {
-        if (job.mode == MODE_RETRIEVE)
-            kvs_ldg_piece_kernel<MODE_RETRIEVE><<<n, kPieceThreads, 0, s>>>(dc);
-        else
-            kvs_ldg_piece_kernel<MODE_STORE><<<n, kPieceThreads, 0, s>>>(dc);
-        return cudaGetLastError();
-    }
     grid = grid > 0 ? clamp_grid(grid, ldg_ctas_per_sm(), job.num_pieces) : (int)job.num_pieces;
-    if (job.mode == MODE_RETRIEVE)
-        kvs_ldg_kernel<V, MODE_RETRIEVE><<<grid, kLdgThreads, 0, s>>>(dc, n);
-    else if (job.mode == MODE_STORE)
-        kvs_ldg_kernel<V, MODE_STORE><<<grid, kLdgThreads, 0, s>>>(dc, n);
-    else
-        kvs_ldg_kernel<V, MODE_COMPARE><<<grid, kLdgThreads, 0, s>>>(dc, n);
+    switch (vec_bytes) {
+        case 16: kvs_compare_kernel<16><<<grid, kLdgThreads, 0, s>>>(dc, n); break;
+        case 8:  kvs_compare_kernel<8><<<grid, kLdgThreads, 0, s>>>(dc, n); break;
+        case 4:  kvs_compare_kernel<4><<<grid, kLdgThreads, 0, s>>>(dc, n); break;
+        case 2:  kvs_compare_kernel<2><<<grid, kLdgThreads, 0, s>>>(dc, n); break;
+        default: kvs_compare_kernel<1><<<grid, kLdgThreads, 0, s>>>(dc, n); break;
+    }
     return cudaGetLastError();
 }
 
@@ -726,8 +1017,12 @@ cudaError_t launch_link_staged(const Job& job, int grid, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t launch_link(const Job& job, int grid, cudaStream_t s) {
+cudaError_t launch_link(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
     if (job.num_pieces == 0) return cudaSuccess;
+    // Short runs as span pieces.  98 MB retrieved in 4 KiB runs: 472 us against 482 by runs, in
+    // 8 KiB runs 474 either way; stored in 4 KiB runs: 534 against 523.
+    if (vec_bytes != 16 || (uint64_t)job.block_size * job.row_bytes < (job.mode == MODE_RETRIEVE ? 8192 : 4096))
+        return launch_spans(job, vec_bytes, clamp_grid(grid, 2, UINT64_MAX), true, s);
     grid = clamp_grid(grid, link_ctas_per_sm(), job.num_pieces);
     const Decoder dc = make_decoder(job);
     const uint32_t n = (uint32_t)job.num_pieces;
@@ -741,7 +1036,7 @@ cudaError_t launch_link(const Job& job, int grid, cudaStream_t s) {
 int ldg_ctas_per_sm() {
     static int n = 0;
     if (n == 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kvs_ldg_kernel<16, MODE_RETRIEVE>, kLdgThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kvs_flat_copy_kernel, kLdgThreads, 0);
         if (n <= 0) n = 1;
         if (n > 4) n = 4;
     }
@@ -750,15 +1045,28 @@ int ldg_ctas_per_sm() {
 
 int tma_ctas_per_sm() { return 1; }
 
+// Chunks in HBM.  Runs of 16 KiB and more at 16-byte alignment, uncapped: one CTA
+// per piece of a run.  Shorter runs, capped grids and odd alignments: span pieces.
+// 12 KiB runs take 173 us as span pieces and 179 as runs (172 by TMA), 16 KiB
+// runs 226.5 us either way, and 20 KiB runs 281.8 us either way.
 cudaError_t launch_ldg(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
     if (job.num_pieces == 0) return cudaSuccess;
-    switch (vec_bytes) {
-        case 16: return launch_ldg_v<16>(job, grid, s);
-        case 8:  return launch_ldg_v<8>(job, grid, s);
-        case 4:  return launch_ldg_v<4>(job, grid, s);
-        case 2:  return launch_ldg_v<2>(job, grid, s);
-        default: return launch_ldg_v<1>(job, grid, s);
+    if (job.mode == MODE_COMPARE) return launch_compare(job, vec_bytes, grid, s);
+    if (vec_bytes == 16 && grid <= 0 && (uint64_t)job.block_size * job.row_bytes >= kPieceBytes / 2) {
+        const Decoder dc = make_decoder(job);
+        const uint32_t n = (uint32_t)job.num_pieces;
+        if (job.mode == MODE_RETRIEVE)
+            kvs_ldg_piece_kernel<MODE_RETRIEVE><<<n, kPieceThreads, 0, s>>>(dc);
+        else
+            kvs_ldg_piece_kernel<MODE_STORE><<<n, kPieceThreads, 0, s>>>(dc);
+        return cudaGetLastError();
     }
+    return launch_spans(job, vec_bytes, grid > 0 ? clamp_grid(grid, kSpanCtasPerSm, job.num_pieces) : 0, false, s);
+}
+
+int kernels_of(const Job& job, int vec_bytes) {
+    const bool runs16 = (uint64_t)job.block_size * job.row_bytes % 16 == 0;
+    return job.mode != MODE_COMPARE && runs16 && has_narrow(job, vec_bytes) ? 2 : 1;
 }
 
 cudaError_t launch_tma(const Job& job, int grid, cudaStream_t s) {

@@ -133,10 +133,11 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     const int L = g->num_layers, B = g->block_size, C = g->chunk_tokens, P = 2 * L;
     const uint64_t R = (uint64_t)g->num_kv_heads * g->head_dim * e_b;
     const uint32_t bpc = (uint32_t)((C + B - 1) / B);
-    uint64_t addr_or = R;
+    uint64_t addr_or = R, span_or = 0;
     for (int p = 0; p < P; ++p) {
         if (!cache->kv_planes[p]) return na_fail(KVS_ERR_INVALID_ARG, "plane %d is NULL", p);
         addr_or |= (uint64_t)cache->kv_planes[p];
+        span_or |= (uint64_t)cache->kv_planes[p];
     }
     uint64_t nent = 0, ndev = 0;
     for (int32_t r = 0; r < nreq; ++r) {
@@ -222,6 +223,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
             int rc = chunk_address(c, r, j, &addr);
             if (rc) return rc;
             addr_or |= addr;
+            span_or |= addr | (uint64_t)c.num_tokens * R;
             entries[e].chunk = addr;
             entries[e].n_tok = c.num_tokens;
             entries[e].pad = 0;
@@ -298,6 +300,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     j.block_size = (uint32_t)B;
     j.pieces_per_run = (uint32_t)ppr;
     j.mode = MODE_RETRIEVE;
+    j.align = (uint32_t)span_or;
     const int cap = (int)KVS_F_GET_MAX_CTAS(flags);
     // host-resident entries: the link kernel on kvs_retrieve's cap (16-byte data)
     const uint32_t nhost = e_host - (uint32_t)ndev;
@@ -307,10 +310,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
         jh.entry_base = (uint32_t)ndev;
         jh.num_entries = nhost;
         jh.num_pieces = (uint64_t)nhost * P * bpc * ppr;
-        if (vec == 16)
-            NA_CUDA(launch_link(jh, cap ? cap : hostlink_grid(true), s));
-        else
-            NA_CUDA(launch_ldg(jh, vec, cap, s));
+        NA_CUDA(launch_link(jh, vec, cap ? cap : hostlink_grid(true), s));
     }
     if (ndev) {
         Job jd = j;
