@@ -369,6 +369,7 @@ int fill_plan(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache,
     }
 
     uint32_t di = 0, hi = pl.num_device;
+    uint32_t tok_device = 0, tok_host = 0;
     for (int32_t r = 0; r < nreq; ++r) {
         const kvs_request& q = reqs[r];
         int64_t s = q.first_token;
@@ -393,7 +394,9 @@ int fill_plan(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache,
             }
             pl.entries[e].chunk = addr;
             pl.entries[e].n_tok = c.num_tokens;
-            pl.entries[e].pad = 0;
+            uint32_t& before = c.residency == KVS_SRC_DEVICE ? tok_device : tok_host;
+            pl.entries[e].first_tok = before;
+            before += (uint32_t)c.num_tokens;
             pl.entry_bytes[e] = (uint64_t)P * c.num_tokens * pl.row_bytes;
             pl.addr_or |= addr;
             pl.span_or |= addr | (uint64_t)c.num_tokens * pl.row_bytes;
@@ -969,6 +972,9 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
         recip(f.job.num_planes * f.job.blocks_per_chunk, f.pe_m, f.pe_p);
         recip(f.job.blocks_per_chunk, f.bpc_m, f.bpc_p);
         f.rows_whole = (kFp8PieceCodes / 16) % (hd / 16) == 0;
+        const Entry& last = pl.entries[first + count - 1];
+        f.tokens = (uint64_t)last.first_tok + (uint32_t)last.n_tok;
+        f.ragged = f.tokens != (uint64_t)count * (uint32_t)g->chunk_tokens;
         return f;
     };
     // store-back segments: one per (chunk, plane, head)

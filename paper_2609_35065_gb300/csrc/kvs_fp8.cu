@@ -35,9 +35,9 @@
 // Store-back to pinned host runs one 256-thread CTA per (chunk, plane, head):
 // the head's BF16 elements are loaded into registers at once, reduced to the
 // amax and quantised from registers (heads too large for that take a two-pass
-// kernel, one CTA per (chunk, plane)).  Into HBM chunks a persistent CTA per SM
-// stages heads in shared memory with per-thread async copies, two heads ahead
-// of the one it quantises.
+// kernel, one CTA per (chunk, plane)).  Into HBM chunks persistent CTAs, two per
+// SM, hold one unit of heads in shared memory and refill it with the next unit's
+// loads while they convert.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -515,44 +515,66 @@ __global__ void __launch_bounds__(kStThreads) kvs_fp8_store_head_kernel(const Fp
 }
 
 // ---------------------------------------------------------------------------
-// Staged store-back for HBM destinations: per-thread async copies
+// Store-back into HBM chunks
 // ---------------------------------------------------------------------------
-// A persistent 512-thread CTA per SM walks segments (as above, one (chunk,
-// plane, head) each).  Thread t owns the 16-byte column w = t % (D/8) of
-// tokens t / (D/8) + u * step, u < kSgVec (step = kSgThreads / (D/8)); its
-// loads go through shared memory: it copies its vectors of segment k with
-// cp.async into its own slots of stage k % kSgStages, kSgStages - 1 segments
-// ahead of the one it quantises, so two heads' loads (128 KiB) are in flight
-// per SM while its registers hold only the current head's 8 vectors.  A thread
-// reads back only the slots it filled itself, so the stages need no CTA
-// barrier (cp.async.wait_group orders them); the amax reduction takes two.
-// Slot u of thread t in a stage is at (u * kSgThreads + t) * 16.  The plane
-// rows of a full segment depend only on its chunk, so a thread keeps them in
-// registers while consecutive segments share the chunk.
-constexpr int kSgThreads = 512;
-constexpr int kSgVec = 8;
-constexpr int kSgStages = 3;
-constexpr uint32_t kSgStageBytes = kSgVec * kSgThreads * 16;        // 64 KiB
-constexpr uint32_t kSgSmemBytes = kSgStages * kSgStageBytes;
-static_assert(kSgStageBytes == kHeadMaxElems * 2, "a stage holds the largest single-pass head");
+// A unit is g heads of one (chunk, plane), held in the shared memory of a persistent
+// 512-thread CTA: thread t owns the 16-byte column w = t % (g * D / 8), which lies in
+// one head, of tokens t / (g * D / 8) + u * step, u < VEC (threads past the last whole
+// row idle), copied by cp.async into slots that only it reads back.  Two passes over
+// the slots: the heads' maxima (one barrier), then conversion; as a slot is converted
+// and its codes are stored, it takes the next unit's vector, so a CTA's loads are in
+// flight while it converts, and two CTAs per SM cover each other's reductions.
+//
+// HBM bounds it (1.5 bytes moved per byte of BF16); what is left to the flat copy's
+// rate is the loads' latency behind the reduction of a unit.  8 requests of the
+// 8B shape (read + write): 2048 tokens 511 -> 495 us (6.5 TB/s), 1900 tokens 482 ->
+// 453 us (6.6 TB/s), against a 512-thread CTA per SM with three 64 KiB stages that
+// split its units evenly.  Tried without gain: three CTAs per SM (507 us), one 256-
+// or 1024-thread shape (+1 to +4%), units in registers with 256-bit loads (497 us),
+// tokens split over clusters of eight so that every access is contiguous (670 us:
+// the cluster barrier and fewer resident CTAs cost more than the pattern; contiguous
+// accesses alone gain 1.5%), bulk copies of 256-byte rows (1170 us: issue rate).
+//
+// VEC = 8 holds 64 KiB a unit, one head of 128 at 256 tokens.  VEC = 13 (104 KiB) is
+// taken where it holds more heads than 8 does: heads of 80 then go in pairs, whose
+// codes are whole sectors (99 -> 89 us; the two-pass kernel took 240), 48 by fours
+// (84 -> 78 us), and one of 192 still fits (147 us; two-pass 429).  Larger heads
+// split their tokens over a cluster, which exchanges maxima (256 tokens of 256: 283
+// -> 108 us), on three CTAs per SM of fewer registers (two: 112 us).
+constexpr int kUqThreads = 512;
+constexpr uint32_t kUqMaxRows = 4096;
+constexpr int kUqVec = 8, kUqVecWide = 13;
+constexpr uint32_t kUqMaxTeam = 8, kUqMaxCluster = 4;
+// What a unit costs beside its bytes (barrier, reduction, latency), in bytes of BF16.
+// 16 x 300 tokens, whose last chunks hold 44: 147 us at 24 KiB, 130 at 128 KiB, 135 at
+// 256; 8 x 1900: 480, 453 and 453.
+constexpr uint32_t kUqUnitBytes = 131072;
+__host__ __device__ constexpr int uq_ctas(bool cluster) { return cluster ? 3 : 2; }
+__host__ __device__ constexpr uint32_t uq_stage_bytes(int vec) { return vec * kUqThreads * 16; }
 
-// A CTA's segments are one contiguous range, walked with a cursor over
-// (entry, plane, head): consecutive segments share the chunk (and its plane
-// rows) and mostly the plane, and need no division to decode.
-struct SgCur {
-    uint32_t e, p, h;
+// CTAs work in teams of G neighbours (G divides the H / g groups of a plane): a
+// team's member m takes groups m, m + G, ... of the same (chunk, plane), so that
+// what the members read of a token row, and write of its codes, lies side by side
+// in memory and moves at the same time (8 x 2048 tokens: teams of 8 504 us, of 1 520).
+// The work of a team is a contiguous range of units (chunk, plane, G groups), walked
+// with a cursor: consecutive units share the chunk and its plane rows, and need no
+// division to decode.  The ranges weigh a unit by its tokens and kUqUnitBytes, so that
+// short last chunks leave no team idle.
+struct UqCur {
+    uint32_t e, p, group;
 };
 
-__device__ __forceinline__ SgCur sg_at(const Fp8Job& f, uint32_t seg) {
+__device__ __forceinline__ UqCur uq_at(const Fp8Job& f, uint32_t unit, uint32_t groups, uint32_t G, uint32_t member) {
     const Job& j = f.job;
-    const uint32_t eh = seg / f.heads, h = seg - eh * f.heads;
-    const uint32_t e = eh / j.num_planes;
-    return {e, j.plane_begin + (eh - e * j.num_planes), h};
+    const uint32_t per = groups / G, eg = unit / per, r = unit - eg * per;
+    const uint32_t e = eg / j.num_planes;
+    return {e, j.plane_begin + (eg - e * j.num_planes), r * G + member};
 }
 
-__device__ __forceinline__ void sg_step(const Fp8Job& f, SgCur& c) {
-    if (++c.h == f.heads) {
-        c.h = 0;
+__device__ __forceinline__ void uq_step(const Fp8Job& f, UqCur& c, uint32_t groups, uint32_t G) {
+    c.group += G;
+    if (c.group >= groups) {
+        c.group -= groups;
         if (++c.p == f.job.plane_begin + f.job.num_planes) {
             c.p = f.job.plane_begin;
             ++c.e;
@@ -564,23 +586,14 @@ __device__ __forceinline__ void cp_async16(uint32_t dst_smem, uint64_t src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst_smem), "l"(src) : "memory");
 }
 
-__device__ __forceinline__ void cp_async_commit() {
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" :: "n"(N) : "memory");
+__device__ __forceinline__ void cp_async_wait_all() {
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 __device__ __forceinline__ uint4 lds16(uint32_t a) {
     uint4 r;
     asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "r"(a));
     return r;
-}
-
-__device__ __forceinline__ void sts16_zero(uint32_t a) {
-    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" :: "r"(a), "r"(0u) : "memory");
 }
 
 // Two BF16 (one word) times `inv` -> two E4M3 codes: two binary32 multiplies
@@ -601,53 +614,6 @@ __device__ __forceinline__ uint2 quant8_pk(const uint4& a, uint64_t inv2) {
                       e4m3x2_of_pk(a.z, inv2) | (e4m3x2_of_pk(a.w, inv2) << 16));
 }
 
-// Plane row (blk * B + token % B) of token i of a chunk, or kNoRow for a bad block.
-constexpr uint32_t kNoRow = 0xFFFFFFFFu;
-
-__device__ __forceinline__ uint32_t sg_row(const Fp8Job& f, const int32_t* blocks, uint32_t i) {
-    const Job& j = f.job;
-    const uint32_t B = j.block_size;
-    const uint32_t bi = B == 1 ? i : __umulhi(i, f.block_magic);
-    const int32_t blk = __ldg(blocks + bi);
-    return (blk < 0 || blk >= j.num_blocks) ? kNoRow : (uint32_t)blk * B + (i - bi * B);
-}
-
-// This thread's loads of segment c (n tokens) into its slots of the stage at
-// `stage`; a bad block's vectors are zeros (and the call reports the error).
-// `rows` / `rows_e`: the cached rows of full segments and the chunk they belong to.
-template <bool FULL>
-__device__ __forceinline__ void sg_issue(const Fp8Job& f, const SgCur& c, uint32_t n, uint32_t stage,
-                                         uint32_t (&rows)[kSgVec], uint32_t& rows_e) {
-    const Job& j = f.job;
-    const uint32_t D = f.head_dim, vpt = D / 8, step = kSgThreads / vpt;
-    const uint32_t w = threadIdx.x % vpt, i0 = threadIdx.x / vpt;
-    const uint64_t row2 = (uint64_t)f.heads * D * 2;
-    const int32_t* blocks = j.blocks + (size_t)(j.entry_base + c.e) * j.blocks_per_chunk;
-    const uint64_t src0 = j.planes[c.p] + (uint64_t)c.h * D * 2 + (uint64_t)w * 16;
-    const uint32_t slot0 = stage + threadIdx.x * 16;
-    if (FULL && rows_e != c.e) {
-#pragma unroll
-        for (int u = 0; u < kSgVec; ++u) rows[u] = sg_row(f, blocks, i0 + u * step);
-        rows_e = c.e;
-    }
-    bool bad = false;
-#pragma unroll
-    for (int u = 0; u < kSgVec; ++u) {
-        const uint32_t i = i0 + u * step;
-        if (FULL || i < n) {
-            const uint32_t row = FULL ? rows[u] : sg_row(f, blocks, i);
-            const uint32_t slot = slot0 + u * kSgThreads * 16;
-            if (row == kNoRow) {
-                bad = true;
-                sts16_zero(slot);
-            } else {
-                cp_async16(slot, src0 + (uint64_t)row * row2);
-            }
-        }
-    }
-    if (bad) atomicCAS(j.err, 0, KVS_ERR_BOUNDS);
-}
-
 // Running max of |x| over BF16 pairs in one instruction (sm_86+): the result's
 // magnitude is the larger magnitude, its sign the XOR of the signs (cleared at
 // the end); a NaN input is ignored.  Infinities are not: a head whose maximum
@@ -660,98 +626,165 @@ __device__ __forceinline__ uint32_t absmax2(uint32_t m2, uint32_t w) {
 
 constexpr uint32_t kBf16Inf = 0x7F80u;
 
-// Quantises segment c (n tokens) from this thread's slots of `stage` (its loads
-// complete).  One barrier: every warp reads all warps' maxima (from the half of
-// warp_max this segment's parity selects) and computes the reciprocal itself;
-// a head holding an infinity takes one more barrier for its finite amax.
-template <bool FULL>
-__device__ __forceinline__ void sg_quantise(const Fp8Job& f, const SgCur& c, uint32_t n, uint32_t stage,
-                                            uint32_t* warp_max, uint32_t* warp_max_fin) {
-    const Job& j = f.job;
-    const uint32_t H = f.heads, D = f.head_dim, vpt = D / 8, step = kSgThreads / vpt;
-    const uint32_t t = threadIdx.x, w = t % vpt, i0 = t / vpt;
-    const uint32_t slot0 = stage + t * 16;
-    uint4 v[kSgVec];
-#pragma unroll
-    for (int u = 0; u < kSgVec; ++u) {
-        v[u] = make_uint4(0, 0, 0, 0);
-        if (FULL || i0 + u * step < n) v[u] = lds16(slot0 + u * kSgThreads * 16);
-    }
-    uint32_t x2 = 0;
-#pragma unroll
-    for (int u = 0; u < kSgVec; ++u)
-        x2 = absmax2(absmax2(absmax2(absmax2(x2, v[u].x), v[u].y), v[u].z), v[u].w);
-    x2 &= 0x7FFF7FFFu;                                      // never NaN: at most kBf16Inf per half
-    uint32_t m = __reduce_max_sync(0xFFFFFFFFu, max(x2 & 0xFFFFu, x2 >> 16));
-    if ((t & 31) == 0) warp_max[t >> 5] = m;
-    __syncthreads();
-    uint32_t a = __reduce_max_sync(0xFFFFFFFFu, warp_max[(t & 31) % (kSgThreads / 32)]);
-    if (a == kBf16Inf) {                                    // uniform across the CTA
-        uint32_t m2 = 0;
-#pragma unroll
-        for (int u = 0; u < kSgVec; ++u)
-            m2 = amax2(amax2(amax2(amax2(m2, v[u].x), v[u].y), v[u].z), v[u].w);
-        m = __reduce_max_sync(0xFFFFFFFFu, amax_bits(m2));
-        if ((t & 31) == 0) warp_max_fin[t >> 5] = m;
-        __syncthreads();
-        a = __reduce_max_sync(0xFFFFFFFFu, warp_max_fin[(t & 31) % (kSgThreads / 32)]);
-    }
-    const float af = __uint_as_float(a << 16);
-    const float inv = af > 0.0f ? __fdiv_rn(448.0f, af) : 1.0f;
-    const uint64_t chunk = j.entries[c.e].chunk;
-    if (t == 0) *reinterpret_cast<float*>(chunk + ((uint64_t)c.p * H + c.h) * 4) = af > 0.0f ? __fdiv_rn(af, 448.0f) : 1.0f;
-    const uint64_t inv2 = ((uint64_t)__float_as_uint(inv) << 32) | __float_as_uint(inv);
-    const uint64_t hd = (uint64_t)H * D;
-    const uint64_t codes = chunk + f.scale_bytes + (uint64_t)c.p * n * hd + (uint64_t)c.h * D + (uint64_t)w * 8 +
-                           (uint64_t)i0 * hd;
-#pragma unroll
-    for (int u = 0; u < kSgVec; ++u)
-        if (FULL || i0 + u * step < n) st_cs8(codes + (uint64_t)(u * step) * hd, quant8_pk(v[u], inv2));
+__device__ __forceinline__ void st_cluster(uint32_t addr, uint32_t rank, uint32_t v) {
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.u32 [%0], %1;" :: "r"(ra), "r"(v) : "memory");
 }
 
-// CTA b takes segments [b * N / G, (b + 1) * N / G).  warp_max has two halves,
-// alternating by segment: a warp writes a half again only two segments later,
-// after the next segment's barrier, which every warp reaches only once it has
-// read this segment's half.  warp_max_fin (heads holding an infinity) is
-// written after a segment's first barrier and read before its next one.
-static_assert(kSgThreads / 32 <= 32, "one lane per warp maximum");
-__global__ void __launch_bounds__(kSgThreads, 1) kvs_fp8_store_staged_kernel(const Fp8Job f, uint32_t num_segments) {
-    extern __shared__ __align__(128) uint8_t sg_stage[];
-    __shared__ uint32_t warp_max[2][kSgThreads / 32];
-    __shared__ uint32_t warp_max_fin[kSgThreads / 32];
-    const uint32_t base = smem_u32(sg_stage);
-    const uint32_t full_n = kSgVec * (kSgThreads / (f.head_dim / 8));
-    const uint32_t lo = (uint32_t)((uint64_t)blockIdx.x * num_segments / gridDim.x);
-    const uint32_t hi = (uint32_t)((uint64_t)(blockIdx.x + 1) * num_segments / gridDim.x);
-    if (lo >= hi) return;                                   // uniform across the CTA
-    const Entry* entries = f.job.entries;
-    uint32_t rows[kSgVec];
-    uint32_t rows_e = 0xFFFFFFFFu;
-    SgCur ic = sg_at(f, lo), qc = ic;                       // issue / quantise cursors
-    uint32_t issued = 0;
-    // one commit group per segment slot, empty past the end, so wait_group counts segments
-    auto issue = [&]() {
-        if (lo + issued < hi) {
-            const uint32_t n = (uint32_t)entries[ic.e].n_tok;
-            const uint32_t stage = base + (issued % kSgStages) * kSgStageBytes;
-            if (n == full_n) sg_issue<true>(f, ic, n, stage, rows, rows_e);
-            else sg_issue<false>(f, ic, n, stage, rows, rows_e);
-            sg_step(f, ic);
-            ++issued;
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// Team k of T takes the units that begin in [k * W / T, (k + 1) * W / T) of the job's
+// W = sum over its chunks of (tokens + extra) x units per chunk.  CLUSTER: the tokens
+// of a unit are split over cl CTAs of a cluster, which exchange their maxima.
+template <int VEC, bool CLUSTER>
+__global__ void __launch_bounds__(kUqThreads, uq_ctas(CLUSTER))
+kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t G, uint32_t extra, uint32_t cl) {
+    extern __shared__ __align__(128) uint8_t uq_smem[];
+    uint32_t* rows = reinterpret_cast<uint32_t*>(uq_smem + uq_stage_bytes(VEC));   // plane row of each of the CTA's tokens
+    // Maxima of unit n's heads in third n % 3, cleared before barrier n - 1: the readers of unit
+    // n - 3 have passed barrier n - 2, and the writers of unit n wait for barrier n - 1.
+    __shared__ uint32_t amax[3][kFp8MaxHeads], exact[kFp8MaxHeads];
+    // The cluster's, by rank, in half n % 2: written before cluster barrier n, read after it, and
+    // written again after cluster barrier n + 1.
+    __shared__ uint32_t all[CLUSTER ? 2 : 1][CLUSTER ? kUqMaxCluster : 1][kFp8MaxHeads];
+    __shared__ uint32_t range[2];
+    const Job& j = f.job;
+    const Entry* entries = j.entries;
+    const uint32_t t = threadIdx.x, D = f.head_dim, vph = D / 8, vpt = g * vph, step = kUqThreads / vpt;
+    const uint32_t w = t % vpt, i0 = t / vpt, hl = w / vph;
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, i0 < step ? hl : 0xFFFFu);   // lanes on the same head
+    const bool lead = i0 < step && (t & 31) == (uint32_t)__ffs(peers) - 1;
+    const uint32_t rank = CLUSTER ? blockIdx.x % cl : 0, unit_cta = CLUSTER ? blockIdx.x / cl : blockIdx.x;
+    const uint32_t groups = f.heads / g, team = unit_cta / G, teams = (CLUSTER ? gridDim.x / cl : gridDim.x) / G;
+    for (uint32_t h = t; h < 3 * kFp8MaxHeads; h += kUqThreads) (&amax[0][0])[h] = 0;
+    const uint32_t upe = j.num_planes * (groups / G);
+    if (f.ragged) {
+        const uint64_t W = (f.tokens + (uint64_t)extra * j.num_entries) * upe;
+        const uint64_t x[2] = {W * team / teams, W * (team + 1) / teams};
+        for (uint32_t e = t; e < j.num_entries; e += kUqThreads) {
+            const uint64_t at = (entries[e].first_tok + (uint64_t)extra * e) * upe;
+            const uint32_t n = (uint32_t)entries[e].n_tok + extra;
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (x[k] >= at && x[k] < at + (uint64_t)n * upe) range[k] = (uint32_t)((uint64_t)e * upe + (x[k] - at + n - 1) / n);
         }
-        cp_async_commit();
-    };
-    for (int s = 0; s + 1 < kSgStages; ++s) issue();
-    for (uint32_t k = 0; lo + k < hi; ++k) {
-        issue();
-        cp_async_wait<kSgStages - 1>();
-        const uint32_t n = (uint32_t)entries[qc.e].n_tok;
-        const uint32_t stage = base + (k % kSgStages) * kSgStageBytes;
-        if (n == full_n) sg_quantise<true>(f, qc, n, stage, warp_max[k & 1], warp_max_fin);
-        else sg_quantise<false>(f, qc, n, stage, warp_max[k & 1], warp_max_fin);
-        sg_step(f, qc);
+        if (t == 0 && x[1] == W) range[1] = j.num_entries * upe;
+    } else if (t < 2) {
+        range[t] = (uint32_t)((uint64_t)j.num_entries * upe * (team + t) / teams);
     }
-    cp_async_wait<0>();
+    if (CLUSTER) cluster_sync();                            // the others have started
+    else __syncthreads();
+    uint32_t left = range[1] - range[0];
+    if (left == 0) return;                                  // uniform across the cluster
+    UqCur c = uq_at(f, range[0], groups, G, unit_cta % G);
+    uint32_t mine = 0, first = 0;                           // the CTA's tokens of the chunk (0 for an idle thread), from `first`
+    // the chunk's plane rows; a block out of range, which the planner has excluded, is reported
+    auto enter = [&]() {
+        const uint32_t n = (uint32_t)entries[c.e].n_tok, B = j.block_size;
+        const int32_t* blocks = j.blocks + (size_t)(j.entry_base + c.e) * j.blocks_per_chunk;
+        const uint32_t per = CLUSTER ? (n + cl - 1) / cl : n;
+        first = CLUSTER ? min(rank * per, n) : 0;
+        const uint32_t count = min(per, n - first);
+        for (uint32_t r = t; r < count; r += kUqThreads) {
+            const uint32_t i = first + r, bi = B == 1 ? i : __umulhi(i, f.block_magic);
+            uint32_t blk = (uint32_t)__ldg(blocks + bi);
+            if (blk >= (uint32_t)j.num_blocks) {
+                atomicCAS(j.err, 0, KVS_ERR_BOUNDS);
+                blk = 0;
+            }
+            rows[r] = blk * B + (i - bi * B);
+        }
+        mine = i0 < step ? count : 0;
+        __syncthreads();
+    };
+    const uint32_t row2 = f.heads * D * 2;
+    auto source = [&]() { return j.planes[c.p] + (uint64_t)(c.group * vpt + w) * 16; };
+    enter();
+    const uint32_t slot0 = smem_u32(uq_smem) + t * 16;      // this thread's vector u at slot0 + u * kUqThreads * 16
+    {
+        const uint64_t src = source();
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+            if (i0 + u * step < mine) cp_async16(slot0 + u * kUqThreads * 16, src + (uint64_t)rows[i0 + u * step] * row2);
+    }
+    for (uint32_t k = 0, half = 0;; half ^= 1) {
+        const uint32_t k1 = k == 2 ? 0 : k + 1;
+        uint32_t x2 = 0;
+        cp_async_wait_all();
+#pragma unroll
+        for (int u = 0; u < VEC; ++u)
+            if (i0 + u * step < mine) {
+                const uint4 v = lds16(slot0 + u * kUqThreads * 16);
+                x2 = absmax2(absmax2(absmax2(absmax2(x2, v.x), v.y), v.z), v.w);
+            }
+        x2 &= 0x7FFF7FFFu;                                  // never NaN: at most kBf16Inf per half
+        const uint32_t m = __reduce_max_sync(peers, max(x2 & 0xFFFFu, x2 >> 16));
+        if (lead) atomicMax(&amax[k][hl], m);
+        if (t < g) amax[k1][t] = 0;
+        __syncthreads();
+        uint32_t a = amax[k][hl];
+        // The maximum over the cluster's CTAs of what each has in own[].
+        auto over_cluster = [&](const uint32_t* own) {
+            for (uint32_t x = t; x < g * cl; x += kUqThreads) st_cluster(smem_u32(&all[half][rank][x % g]), x / g, own[x % g]);
+            cluster_sync();
+            uint32_t r = 0;
+            for (uint32_t c2 = 0; c2 < cl; ++c2) r = max(r, all[half][c2][hl]);
+            return r;
+        };
+        if (CLUSTER) a = over_cluster(amax[k]);
+        // a head with an infinity: the largest finite magnitudes of the unit's heads instead
+        uint32_t top = 0;                                   // uniform across the cluster
+        if (g == 1) top = a;
+        else for (uint32_t x = t & 31; x < g; x += 32) top = max(top, amax[k][x]);   // a cluster has one head a unit
+        if (g > 1) top = __reduce_max_sync(0xFFFFFFFFu, top);
+        if (top == kBf16Inf) {
+            uint32_t m2 = 0;
+            for (int u = 0; u < VEC; ++u)
+                if (i0 + u * step < mine) {
+                    const uint4 v = lds16(slot0 + u * kUqThreads * 16);
+                    m2 = amax2(amax2(amax2(amax2(m2, v.x), v.y), v.z), v.w);
+                }
+            const uint32_t mf = __reduce_max_sync(peers, amax_bits(m2));
+            if (t < g) exact[t] = 0;
+            __syncthreads();
+            if (lead) atomicMax(&exact[hl], mf);
+            __syncthreads();
+            a = exact[hl];
+            if (CLUSTER) {
+                cluster_sync();                             // the first maxima have been read
+                a = over_cluster(exact);
+            }
+        }
+        const float af = __uint_as_float(a << 16);
+        const float inv = af > 0.0f ? __fdiv_rn(448.0f, af) : 1.0f;
+        const Entry en = entries[c.e];
+        const uint32_t h0 = c.group * g, hd = f.heads * D, old = mine;
+        if (rank == 0 && i0 == 0 && w % vph == 0)
+            reinterpret_cast<float*>(en.chunk)[(uint64_t)c.p * f.heads + h0 + hl] = af > 0.0f ? __fdiv_rn(af, 448.0f) : 1.0f;
+        const uint64_t codes = en.chunk + f.scale_bytes + ((uint64_t)c.p * (uint32_t)en.n_tok + first + i0) * hd + (uint64_t)h0 * D + w * 8;
+        uint64_t src = 0;
+        if (--left) {
+            const uint32_t e = c.e;
+            uq_step(f, c, groups, G);
+            if (c.e != e) enter();                          // every thread has used the old rows
+            src = source();
+        } else {
+            mine = 0;
+        }
+        const uint64_t inv2 = ((uint64_t)__float_as_uint(inv) << 32) | __float_as_uint(inv);
+#pragma unroll
+        for (int u = 0; u < VEC; ++u) {
+            const uint32_t i = i0 + u * step;
+            if (i < old)
+                st_cs8(codes + (uint64_t)(u * step) * hd, quant8_pk(lds16(slot0 + u * kUqThreads * 16), inv2));
+            if (i < mine) cp_async16(slot0 + u * kUqThreads * 16, src + (uint64_t)rows[i] * row2);
+        }
+        if (!left) break;
+        k = k1;
+    }
 }
 
 constexpr int kStUnroll = 4;                         // vectors per thread in flight per step
@@ -854,7 +887,6 @@ __global__ void __launch_bounds__(kStThreads) kvs_fp8_store_kernel(const Fp8Job 
 
 constexpr int kMaxDev = 64;
 int g_sms[kMaxDev];                      // SM count per device
-bool g_sg_attr[kMaxDev];                 // dynamic shared memory limit of the staged store raised
 bool g_fs_attr[kMaxDev];                 // ... of the few-SM retrieval
 
 int sm_count() {
@@ -908,28 +940,87 @@ cudaError_t launch_fp8_retrieve_staged(const Fp8Job& fj, int grid, cudaStream_t 
     return cudaGetLastError();
 }
 
+// Team size: the divisor of the groups that leaves the fewest CTAs of the grid without a
+// team; the larger among equals, kUqMaxTeam at most.
+uint32_t uq_team(uint32_t groups, uint32_t ctas) {
+    uint32_t best = 1;
+    for (uint32_t n = 2; n <= kUqMaxTeam && n <= ctas; ++n)
+        if (groups % n == 0 && ctas % n <= ctas % best) best = n;
+    return best;
+}
+
+// Heads per unit: the most whose tokens fit the vectors of one CTA; 0 where one head does not.
+uint32_t uq_heads(const Fp8Job& fj, uint32_t chunk_tokens, uint32_t vec) {
+    for (uint32_t g = fj.heads; g >= 1; --g) {
+        const uint32_t vpt = g * (fj.head_dim / 8);
+        if (fj.heads % g == 0 && vpt <= kUqThreads && vec * (kUqThreads / vpt) >= chunk_tokens) return g;
+    }
+    return 0;
+}
+
+template <int VEC, bool CLUSTER>
+cudaError_t launch_unit(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chunk_tokens, uint32_t g, uint32_t cl) {
+    if (fj.job.num_entries == 0) return cudaSuccess;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= kMaxDev) dev = 0;
+    const auto k = kvs_fp8_store_unit_kernel<VEC, CLUSTER>;
+    static bool attr[kMaxDev];                              // shared-memory limit raised
+    if (!attr[dev]) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)(uq_stage_bytes(VEC) + kUqMaxRows * 4));
+        if (e != cudaSuccess) return e;
+        attr[dev] = true;
+    }
+    int full = sm_count() * uq_ctas(CLUSTER) / (int)cl;
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(kUqThreads);
+    cfg.dynamicSmemBytes = uq_stage_bytes(VEC) + (chunk_tokens + cl - 1) / cl * 4;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    if (CLUSTER) {                                          // as many clusters as the GPCs hold at once
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = cl;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        cfg.gridDim = dim3((uint32_t)full * cl);
+        int most = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&most, k, &cfg);
+        if (e != cudaSuccess) return e;
+        full = std::max(1, std::min(full, most));
+    }
+    int ctas = grid > 0 ? std::max(1, std::min(grid / (int)cl, full)) : full;
+    uint64_t units = 0;
+    for (;; --g) {                                          // fewer heads a unit while CTAs have none
+        if (fj.heads % g) continue;
+        units = (uint64_t)fj.job.num_entries * fj.job.num_planes * (fj.heads / g);
+        if (g == 1 || units >= (uint64_t)ctas) break;
+    }
+    if ((uint64_t)ctas > units) ctas = (int)units;
+    const uint32_t G = uq_team(fj.heads / g, (uint32_t)ctas);
+    cfg.gridDim = dim3((uint32_t)ctas / G * G * cl);
+    const uint32_t extra = kUqUnitBytes / (g * fj.head_dim * 2);
+    return cudaLaunchKernelEx(&cfg, k, fj, g, G, extra, cl);
+}
+
 cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chunk_tokens, bool staged) {
     const uint32_t vpt = fj.head_dim / 8;
+    // HBM destinations: plane rows below 2^32, block numbers by a reciprocal (chunk and block
+    // sizes below 2^16), a row table of at most 16 KiB.
+    if (staged && chunk_tokens <= kUqMaxRows && (uint64_t)fj.job.num_blocks * fj.job.block_size <= 0xFFFFFFFFull) {
+        const uint32_t g = uq_heads(fj, chunk_tokens, kUqVec), gw = uq_heads(fj, chunk_tokens, kUqVecWide);
+        if (gw > g) return launch_unit<kUqVecWide, false>(fj, grid, s, chunk_tokens, gw, 1);
+        if (g) return launch_unit<kUqVec, false>(fj, grid, s, chunk_tokens, g, 1);
+        uint32_t cl = 2;
+        while (cl <= kUqMaxCluster && vpt <= kUqThreads && kUqVec * (kUqThreads / vpt) * cl < chunk_tokens) cl *= 2;
+        if (cl <= kUqMaxCluster && vpt <= kUqThreads && (grid <= 0 || grid >= (int)cl))
+            return launch_unit<kUqVec, true>(fj, grid, s, chunk_tokens, 1, cl);
+    }
     if ((uint64_t)chunk_tokens * fj.head_dim <= kHeadMaxElems && kStThreads % vpt == 0 && chunk_tokens < 65536 &&
         fj.job.block_size < 65536) {
         const uint64_t segs = (uint64_t)fj.job.num_entries * fj.job.num_planes * fj.heads;
         if (segs == 0) return cudaSuccess;
-        // the staged kernel needs D/8 to divide its CTA and plane rows below 2^32 - 1
-        if (staged && kSgThreads % vpt == 0 && (uint64_t)fj.job.num_blocks * fj.job.block_size < 0xFFFFFFFFull) {
-            int dev = 0;
-            cudaGetDevice(&dev);
-            if (dev < 0 || dev >= kMaxDev) dev = 0;
-            if (!g_sg_attr[dev]) {
-                const cudaError_t e = cudaFuncSetAttribute(kvs_fp8_store_staged_kernel,
-                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, kSgSmemBytes);
-                if (e != cudaSuccess) return e;
-                g_sg_attr[dev] = true;
-            }
-            if (grid <= 0 || grid > sm_count()) grid = sm_count();
-            if ((uint64_t)grid > segs) grid = (int)segs;
-            kvs_fp8_store_staged_kernel<<<grid, kSgThreads, kSgSmemBytes, s>>>(fj, (uint32_t)segs);
-            return cudaGetLastError();
-        }
         if (grid <= 0 || (uint64_t)grid > segs) grid = (int)std::min<uint64_t>(segs, 1u << 30);
         kvs_fp8_store_head_kernel<<<grid, kStThreads, 0, s>>>(fj, (uint32_t)segs);
         return cudaGetLastError();

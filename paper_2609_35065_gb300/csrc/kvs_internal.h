@@ -13,7 +13,7 @@ namespace kvs {
 struct Entry {
     uint64_t chunk;     // device-visible address of the chunk buffer
     int32_t  n_tok;     // tokens held by the chunk (its token stride)
-    int32_t  pad;
+    uint32_t first_tok; // tokens of the earlier entries of its class (device or host chunks)
 };
 static_assert(sizeof(Entry) == 16, "Entry is uploaded as raw bytes");
 
@@ -96,6 +96,8 @@ struct Fp8Job {
     // entry (num_planes * blocks_per_chunk) and blocks per chunk.
     uint32_t ppr_m, ppr_p, pe_m, pe_p, bpc_m, bpc_p;
     uint32_t rows_whole;         // 1 when every piece starts at a token row (H*D/16 divides 1024)
+    uint64_t tokens;             // of all entries of the job
+    uint32_t ragged;             // 1 when some entry holds fewer tokens than another
 };
 constexpr uint32_t kFp8MaxHeads = 128;
 // Retrieval: a persistent grid of `grid` CTAs (<= 0: fill the GPU) over pieces of at
@@ -110,8 +112,8 @@ cudaError_t launch_fp8_retrieve_staged(const Fp8Job& fj, int grid, cudaStream_t 
 // Store-back: one CTA per (entry, plane, head) in a single pass when a head's
 // chunk_tokens x head_dim elements fit the CTA's registers, else one CTA per
 // (entry, plane) in two passes; a grid-stride loop over them with `grid` > 0.
-// `staged` (HBM destinations): the single pass runs as a persistent CTA per SM
-// (at most `grid` > 0) that stages heads in shared memory with bulk copies.
+// `staged` (HBM destinations): persistent CTAs (at most `grid` > 0) that hold a unit of
+// heads, or with a cluster a part of one, in shared memory.
 cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chunk_tokens, bool staged);
 // Codes per retrieval piece (16 KiB).
 constexpr uint32_t kFp8PieceCodes = 16384;

@@ -226,7 +226,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
             span_or |= addr | (uint64_t)c.num_tokens * R;
             entries[e].chunk = addr;
             entries[e].n_tok = c.num_tokens;
-            entries[e].pad = 0;
+            entries[e].first_tok = 0;                   // read by the fp8 store-back only
             for (uint32_t i = 0; i < bpc; ++i) {
                 const uint32_t ref = e * bpc + i;
                 blocks[ref] = -1;
