@@ -24,14 +24,11 @@
 // both signs and compares with the oracle).
 //
 // Retrieval is bound by the host link (or HBM for device chunks): a persistent
-// grid of 128-thread CTAs walks 16 KiB pieces of codes; each thread keeps two
-// pieces' worth of 16-byte code vectors in registers, so the next piece's
-// loads are in flight while the current one is converted and stored.  The H
-// scales of a piece's plane are loaded once per piece by H threads (one 4-byte
-// load each, beside the codes) and shared through shared memory, instead of
-// one scale load per vector; HBM chunks run one CTA per piece instead, and
-// KVS_F_FEW_SMS runs a kernel that also stages pieces in shared memory so
-// that fewer SMs hold the link beside other kernels.
+// grid of 256-thread CTAs walks span pieces of 16 KiB of codes; each thread keeps two
+// pieces' worth of 16-byte code vectors in registers, so the next piece's loads
+// are in flight while the current one is converted and stored.  HBM chunks run one
+// CTA per piece instead, and KVS_F_FEW_SMS runs a kernel that also stages pieces in
+// shared memory so that fewer SMs hold the link beside other kernels.
 // Store-back to pinned host runs one 256-thread CTA per (chunk, plane, head):
 // the head's BF16 elements are loaded into registers at once, reduced to the
 // amax and quantised from registers (heads too large for that take a two-pass
@@ -48,13 +45,17 @@
 #include "kvs.h"
 #include "kvs_async.cuh"
 #include "kvs_internal.h"
+#include "kvs_job.cuh"
 
 namespace kvs {
 namespace {
 
-constexpr int kRtThreads = 128;
-constexpr int kRtVec = 8;                            // 16-code vectors per thread per piece
-static_assert(kRtThreads * kRtVec * 16 == kFp8PieceCodes, "a piece is one vector set per CTA");
+// Threads, 16-code vectors per thread per piece, and CTAs per SM of the retrieval
+// kernels: host chunks (two pieces in registers each), HBM chunks.
+constexpr int kRtLink = 256, kRtLinkVec = 4, kRtLinkCtas = 4;
+constexpr int kRtHbm = 256, kRtHbmVec = 4, kRtHbmCtas = 6;
+static_assert(kRtLink * kRtLinkVec * 16 == kFp8PieceCodes && kRtHbm * kRtHbmVec * 16 == kFp8PieceCodes,
+              "a piece is one vector set per CTA");
 constexpr int kStThreads = 256;
 
 struct Fp8Piece {
@@ -71,19 +72,15 @@ __device__ __forceinline__ uint32_t fp8_div(uint32_t n, uint32_t m, uint32_t p) 
     return (uint32_t)(((uint64_t)n * m) >> p);
 }
 
-// FAST: the reciprocal divisions (persistent kernels decode a piece per loop
-// trip); the one-piece-per-CTA kernel keeps plain divisions and per-vector head indices,
-// which holds it at fewer registers.
-template <bool FAST = true>
 __device__ __forceinline__ bool fp8_piece(const Fp8Job& f, uint32_t q, Fp8Piece& pc) {
     const Job& j = f.job;
     const uint32_t hd = f.heads * f.head_dim;
     const uint32_t per_entry = j.num_planes * j.blocks_per_chunk;
-    const uint32_t run = FAST ? fp8_div(q, f.ppr_m, f.ppr_p) : q / j.pieces_per_run;
+    const uint32_t run = fp8_div(q, f.ppr_m, f.ppr_p);
     const uint32_t k = q - run * j.pieces_per_run;
-    const uint32_t e = FAST ? fp8_div(run, f.pe_m, f.pe_p) : run / per_entry;
+    const uint32_t e = fp8_div(run, f.pe_m, f.pe_p);
     const uint32_t rem = run - e * per_entry;
-    const uint32_t pr = FAST ? fp8_div(rem, f.bpc_m, f.bpc_p) : rem / j.blocks_per_chunk;
+    const uint32_t pr = fp8_div(rem, f.bpc_m, f.bpc_p);
     const uint32_t i = rem - pr * j.blocks_per_chunk;
     const uint32_t p = j.plane_begin + pr;
     const int32_t blk = __ldg(j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i);
@@ -141,28 +138,182 @@ __device__ __forceinline__ void dequant16(const uint4& c, float s, uint4& lo, ui
     hi.w = e4m3x2_to_bf16x2(c.w >> 16, s);
 }
 
-// A piece's codes in registers; thread t < H also holds the scale of head t,
-// loaded once per piece (not once per vector) beside the codes.
-struct RtRegs {
-    uint4 c[kRtVec];
-    float s;
+// ---------------------------------------------------------------------------
+// Span pieces, as for BF16 copies: piece_codes of the contiguous codes of one
+// (chunk, plane), whatever block boundaries they meet, so that short runs (few KV
+// heads, small blocks) still fill a CTA.  Offsets are in codes.  One run a piece
+// before: 8000 tokens x 24 layers in runs of 2 KiB of codes 42 -> 27.5 us from HBM
+// and 293 -> 241 us from the host (the link's own time: 233), in 512-byte runs 58 ->
+// 16.6 and 480 -> 124.5 us.
+// ---------------------------------------------------------------------------
+struct Fp8Spans {
+    Fp8Job   f;
+    FastDiv  spp, planes, run;      // pieces per span of a full chunk, planes, run codes B*H*D
+    FastDiv  vpr, vph;              // 16-code vectors per token row, and per head
+    uint64_t run_codes;
+    uint32_t piece_codes, num_pieces;
+    uint32_t long_runs;             // runs longer than a piece: a piece meets at most two
+    uint32_t far_spans;             // spans of 2^31 codes or more: divide in 64 bits
 };
 
-__device__ __forceinline__ void rt_load(const Fp8Job& f, const Fp8Piece& pc, RtRegs& r) {
-    const uint32_t nv = pc.len / 16;
-#pragma unroll
-    for (int u = 0; u < kRtVec; ++u) {
-        const uint32_t v = threadIdx.x + u * kRtThreads;
-        if (v < nv) r.c[u] = ld_nc16(pc.codes + (uint64_t)v * 16);
+struct Fp8Span {
+    uint64_t       codes;           // first code of the piece
+    uint64_t       plane;           // base of the plane; long runs: plus the first code's offset in its run
+    uint64_t       scales;          // H binary32 of the plane
+    const int32_t* blocks;          // physical block of the run that holds the first code, and on
+    uint32_t       off;             // short runs: offset of the first code in its run; long runs:
+                                    // codes from it to the end of its run, at most piece_codes
+    uint32_t       len;             // codes, a multiple of 16
+    uint32_t       col;             // column of the first vector in its token row
+};
+
+// Piece q; false for pieces past the end of a short chunk.  Uniform across the CTA.
+__device__ __forceinline__ bool fp8_span(const Fp8Spans& dc, uint32_t q, Fp8Span& sp) {
+    const Job& j = dc.f.job;
+    const uint32_t ep = fdiv(q, dc.spp), k = q - ep * dc.spp.d, e = fdiv(ep, dc.planes);
+    const uint32_t p = j.plane_begin + (ep - e * dc.planes.d);
+    const uint64_t at = (uint64_t)k * dc.piece_codes;
+    uint64_t i0, row;
+    if (dc.far_spans) {
+        i0 = at / dc.run_codes;
+        row = at / 16 / dc.vpr.d;
+    } else {
+        i0 = fdiv((uint32_t)at, dc.run);
+        row = fdiv((uint32_t)at / 16, dc.vpr);
     }
-    if (threadIdx.x < f.heads) r.s = __ldg(reinterpret_cast<const float*>(pc.scales) + threadIdx.x);
+    const Entry en = j.entries[e];
+    const uint64_t span = (uint64_t)en.n_tok * (dc.f.heads * dc.f.head_dim);
+    if (at >= span) return false;
+    const uint64_t off = at - i0 * dc.run_codes;
+    sp.len = (uint32_t)min((uint64_t)dc.piece_codes, span - at);
+    sp.col = (uint32_t)(at / 16 - row * dc.vpr.d);
+    sp.codes = en.chunk + dc.f.scale_bytes + (uint64_t)p * span + at;
+    sp.scales = en.chunk + (uint64_t)p * dc.f.heads * 4;
+    sp.plane = j.planes[p] + (dc.long_runs ? off * 2 : 0);
+    sp.blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i0;
+    sp.off = (uint32_t)(dc.long_runs ? min(dc.run_codes - off, (uint64_t)dc.piece_codes) : off);
+    return true;
 }
 
-// Publishes the piece's scales in shared memory (after every thread has finished
-// with the previous piece's), then converts and stores this thread's vectors.
-// Head of this thread's vector v of a piece: when pieces start at token rows
-// and a row's vpr vectors divide the CTA's thread count T, vector tid + u*T
-// is always in head (tid % vpr) / vph, computed once per thread (`h_fixed`).
+// Run of code x, counted from the piece's first; its block's BF16 address of code x.
+__device__ __forceinline__ uint32_t fp8_run(const Fp8Spans& dc, const Fp8Span& sp, uint32_t x) {
+    return dc.long_runs ? (uint32_t)(x >= sp.off) : fdiv(sp.off + x, dc.run);
+}
+
+__device__ __forceinline__ uint64_t fp8_plane(const Fp8Spans& dc, const Fp8Span& sp, uint32_t x, int32_t blk) {
+    const uint32_t i = fp8_run(dc, sp, x);
+    if (dc.long_runs) return sp.plane + ((uint64_t)((int64_t)blk - (int64_t)i) * dc.run_codes + x) * 2;
+    return sp.plane + ((uint64_t)(uint32_t)blk * dc.run_codes + (sp.off + x - i * (uint32_t)dc.run_codes)) * 2;
+}
+
+// Head of vector v of a piece.
+__device__ __forceinline__ uint32_t fp8_vec_head(const Fp8Spans& dc, const Fp8Span& sp, uint32_t v) {
+    const uint32_t c = sp.col + v;
+    return fdiv(c - fdiv(c, dc.vpr) * dc.vpr.d, dc.vph);
+}
+
+// A vector's 32 bytes of BF16 at `a` (0: nowhere), every lane of the warp together.
+// Two 16-byte stores at a lane stride of 32 bytes would each write half of every
+// sector, so neighbouring lanes swap halves and each store writes whole sectors.  8B
+// shape, 8192 tokens from HBM: 268 us unswapped, 236 swapped (6.8 TB/s read + write);
+// 256-bit stores, which need 32-byte aligned planes, take 239.
+__device__ __forceinline__ void st_bf16x16(uint64_t a, const uint4& lo, const uint4& hi) {
+    const bool odd = threadIdx.x & 1;
+    const uint64_t b = __shfl_xor_sync(0xFFFFFFFFu, a, 1);
+    uint4 x = odd ? lo : hi;
+    x.x = __shfl_xor_sync(0xFFFFFFFFu, x.x, 1);
+    x.y = __shfl_xor_sync(0xFFFFFFFFu, x.y, 1);
+    x.z = __shfl_xor_sync(0xFFFFFFFFu, x.z, 1);
+    x.w = __shfl_xor_sync(0xFFFFFFFFu, x.w, 1);
+    const uint64_t first = odd ? b : a, second = odd ? a : b;   // the even lane's vector, the odd one's
+    if (first) st_cs16(first + (odd ? 16 : 0), odd ? x : lo);
+    if (second) st_cs16(second + (odd ? 16 : 0), odd ? hi : x);
+}
+
+// This thread's vectors of a piece in flight: codes, the scales of their heads, blocks
+// (-1: no such vector; one out of range, which the planner has excluded, is reported).
+template <int U>
+struct RtRegs {
+    uint4   c[U];
+    float   s[U];
+    int32_t blk[U];
+};
+
+template <int T, int U>
+__device__ __forceinline__ void rt_load(const Fp8Spans& dc, const Fp8Span& sp, RtRegs<U>& r) {
+    const uint32_t nv = sp.len / 16;
+    bool bad = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const uint32_t v = threadIdx.x + u * T;
+        if (v < nv) r.c[u] = ld_nc16(sp.codes + (uint64_t)v * 16);
+        r.s[u] = __ldg(reinterpret_cast<const float*>(sp.scales) + fp8_vec_head(dc, sp, min(v, nv - 1)));
+        r.blk[u] = __ldg(sp.blocks + fp8_run(dc, sp, min(v, nv - 1) * 16));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const bool in = (uint32_t)r.blk[u] < (uint32_t)dc.f.job.num_blocks;
+        bad |= !in && r.blk[u] >= 0;
+        if (!in || threadIdx.x + u * T >= nv) r.blk[u] = -1;
+    }
+    if (bad) atomicCAS(dc.f.job.err, 0, KVS_ERR_BOUNDS);
+}
+
+// Every thread of the CTA, converting and storing.
+template <int T, int U>
+__device__ __forceinline__ void rt_store(const Fp8Spans& dc, const Fp8Span& sp, const RtRegs<U>& r) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        uint4 lo, hi;
+        dequant16(r.c[u], r.s[u], lo, hi);
+        st_bf16x16(r.blk[u] < 0 ? 0 : fp8_plane(dc, sp, (threadIdx.x + u * T) * 16, r.blk[u]), lo, hi);
+    }
+}
+
+__device__ __forceinline__ bool rt_next(const Fp8Spans& dc, uint32_t& q, Fp8Span& sp) {
+    while (q < dc.num_pieces) {
+        const uint32_t cur = q;
+        q += gridDim.x;
+        if (fp8_span(dc, cur, sp)) return true;
+    }
+    return false;
+}
+
+// Host chunks: the next piece's loads are in flight while a piece is converted.  64
+// registers, so that four CTAs, 128 KiB of codes, still share an SM beside a kernel
+// that leaves them few SMs.  8192 tokens of the 8B shape: 2561 us with 128 threads x
+// 8 vectors and scales through shared memory, 2570 without it, 2555 here (the link:
+// 2541); 512 x 2 gains another 0.1% but fits two CTAs per SM.
+__global__ void __launch_bounds__(kRtLink, kRtLinkCtas) kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc) {
+    RtRegs<kRtLinkVec> ra, rb;
+    Fp8Span pa, pb;
+    uint32_t q = blockIdx.x;
+    bool ha = rt_next(dc, q, pa);
+    if (ha) rt_load<kRtLink>(dc, pa, ra);
+    while (ha) {
+        const bool hb = rt_next(dc, q, pb);
+        if (hb) rt_load<kRtLink>(dc, pb, rb);
+        rt_store<kRtLink>(dc, pa, ra);
+        if (!hb) break;
+        ha = rt_next(dc, q, pa);
+        if (ha) rt_load<kRtLink>(dc, pa, ra);
+        rt_store<kRtLink>(dc, pb, rb);
+    }
+}
+
+// HBM chunks: one CTA per piece, no persistence; six CTAs per SM (four, or 128 threads x 8
+// vectors, or 512 x 2: up to 1% slower).
+__global__ void __launch_bounds__(kRtHbm, kRtHbmCtas) kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc) {
+    Fp8Span sp;
+    if (!fp8_span(dc, blockIdx.x, sp)) return;              // uniform across the CTA
+    RtRegs<kRtHbmVec> r;
+    rt_load<kRtHbm>(dc, sp, r);
+    rt_store<kRtHbm>(dc, sp, r);
+}
+
+// Head of this thread's vector v of a piece of one run: when pieces start at token
+// rows and a row's vpr vectors divide the CTA's thread count T, vector tid + u*T is
+// always in head (tid % vpr) / vph, computed once per thread (`h_fixed`).
 __device__ __forceinline__ uint32_t fp8_fixed_head(const Fp8Job& f, uint32_t T) {
     const uint32_t vph = f.head_dim / 16, vpr = f.heads * vph;
     return (f.rows_whole && T % vpr == 0) ? (threadIdx.x % vpr) / vph : 0xFFFFFFFFu;
@@ -174,24 +325,6 @@ __device__ __forceinline__ uint32_t fp8_head(const Fp8Job& f, const Fp8Piece& pc
     return ((pc.vec0 + v) % vpr) / vph;
 }
 
-__device__ __forceinline__ void rt_store(const Fp8Job& f, const Fp8Piece& pc, const RtRegs& r, float* sm_scale,
-                                         uint32_t h_fixed) {
-    const uint32_t nv = pc.len / 16;
-    __syncthreads();
-    if (threadIdx.x < f.heads) sm_scale[threadIdx.x] = r.s;
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < kRtVec; ++u) {
-        const uint32_t v = threadIdx.x + u * kRtThreads;
-        if (v < nv) {
-            uint4 lo, hi;
-            dequant16(r.c[u], sm_scale[fp8_head(f, pc, v, h_fixed)], lo, hi);
-            st_cs16(pc.out + (uint64_t)v * 32, lo);
-            st_cs16(pc.out + (uint64_t)v * 32 + 16, hi);
-        }
-    }
-}
-
 __device__ __forceinline__ bool rt_next(const Fp8Job& f, uint32_t n, uint32_t& q, Fp8Piece& pc) {
     while (q < n) {
         const uint32_t cur = q;
@@ -199,40 +332,6 @@ __device__ __forceinline__ bool rt_next(const Fp8Job& f, uint32_t n, uint32_t& q
         if (fp8_piece(f, cur, pc)) return true;
     }
     return false;
-}
-
-// Every thread of a CTA walks the same sequence of pieces (the piece index
-// depends only on blockIdx), so the barriers in rt_store are reached by all.
-__global__ void __launch_bounds__(kRtThreads) kvs_fp8_retrieve_kernel(const Fp8Job f, uint32_t num_pieces) {
-    __shared__ float sm_scale[kFp8MaxHeads];
-    const uint32_t h_fixed = fp8_fixed_head(f, kRtThreads);
-    RtRegs ra, rb;
-    Fp8Piece pa, pb;
-    uint32_t q = blockIdx.x;
-    bool ha = rt_next(f, num_pieces, q, pa);
-    if (ha) rt_load(f, pa, ra);
-    while (ha) {
-        const bool hb = rt_next(f, num_pieces, q, pb);
-        if (hb) rt_load(f, pb, rb);
-        rt_store(f, pa, ra, sm_scale, h_fixed);
-        if (!hb) break;
-        ha = rt_next(f, num_pieces, q, pa);
-        if (ha) rt_load(f, pa, ra);
-        rt_store(f, pb, rb, sm_scale, h_fixed);
-    }
-}
-
-// Device chunks (HBM source): one CTA per piece, no persistence; the launch
-// bound keeps the kernel at 64 registers so eight CTAs -- 128 KiB of code
-// loads -- are in flight per SM, and the hardware block scheduler overlaps one
-// CTA's stores with the next CTA's loads.
-__global__ void __launch_bounds__(kRtThreads, 8) kvs_fp8_retrieve_piece_kernel(const Fp8Job f) {
-    __shared__ float sm_scale[kFp8MaxHeads];
-    Fp8Piece pc;
-    if (!fp8_piece<false>(f, blockIdx.x, pc)) return;  // uniform across the CTA
-    RtRegs r;
-    rt_load(f, pc, r);
-    rt_store(f, pc, r, sm_scale, 0xFFFFFFFFu);
 }
 
 // Few-SM flavour of the host-chunk retrieval (KVS_F_FEW_SMS): the scheme of
@@ -903,19 +1002,38 @@ int sm_count() {
 
 }  // namespace
 
+Fp8Spans make_spans(const Fp8Job& fj, uint32_t piece_codes) {
+    Fp8Spans dc;
+    const uint32_t hd = fj.heads * fj.head_dim;
+    dc.f = fj;
+    dc.piece_codes = piece_codes;
+    dc.run_codes = (uint64_t)fj.job.block_size * hd;
+    const uint64_t span = dc.run_codes * fj.job.blocks_per_chunk;          // of a full chunk
+    dc.spp = make_fastdiv((uint32_t)((span + piece_codes - 1) / piece_codes));
+    dc.planes = make_fastdiv(fj.job.num_planes);
+    dc.run = make_fastdiv(dc.run_codes < (1ull << 31) ? (uint32_t)dc.run_codes : 1u);      // longer: never divided by
+    dc.vpr = make_fastdiv(hd / 16);
+    dc.vph = make_fastdiv(fj.head_dim / 16);
+    dc.long_runs = dc.run_codes > piece_codes;
+    dc.far_spans = span >= (1ull << 31);
+    dc.num_pieces = (uint32_t)((uint64_t)fj.job.num_entries * fj.job.num_planes * dc.spp.d);
+    return dc;
+}
+
 cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s) {
-    const uint64_t n = fj.job.num_pieces;
-    if (n == 0) return cudaSuccess;
-    if (grid == kFp8PerPiece) {
-        kvs_fp8_retrieve_piece_kernel<<<(uint32_t)n, kRtThreads, 0, s>>>(fj);
-        return cudaGetLastError();
-    }
-    int per_sm = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kvs_fp8_retrieve_kernel, kRtThreads, 0);
-    const int full = sm_count() * std::max(per_sm, 1);
-    if (grid <= 0 || grid > full) grid = full;
-    if ((uint64_t)grid > n) grid = (int)n;
-    kvs_fp8_retrieve_kernel<<<grid, kRtThreads, 0, s>>>(fj, (uint32_t)n);
+    if (fj.job.num_pieces == 0) return cudaSuccess;
+    const bool per_piece = grid == kFp8PerPiece;
+    const uint32_t vpr = fj.heads * fj.head_dim / 16;
+    // 16 KiB of codes a piece, halved while a launch would leave CTAs without one, down to 4 KiB
+    const int full = sm_count() * kRtLinkCtas;
+    if (!per_piece && (grid <= 0 || grid > full)) grid = full;
+    const uint64_t total = (uint64_t)fj.job.num_entries * fj.job.num_planes * fj.job.blocks_per_chunk * fj.job.block_size * vpr * 16;
+    uint32_t piece = kFp8PieceCodes;
+    while (piece > kFp8PieceCodes / 4 && total / piece < 2ull * (per_piece ? sm_count() : grid)) piece /= 2;
+    const Fp8Spans dc = make_spans(fj, piece);
+    const uint32_t ctas = per_piece ? dc.num_pieces : std::min<uint32_t>((uint32_t)grid, dc.num_pieces);
+    if (per_piece) kvs_fp8_retrieve_piece_kernel<<<ctas, kRtHbm, 0, s>>>(dc);
+    else kvs_fp8_retrieve_kernel<<<ctas, kRtLink, 0, s>>>(dc);
     return cudaGetLastError();
 }
 
