@@ -4,8 +4,8 @@
 // A call is planned on the host: every (request, chunk) pair becomes one
 // Entry, every block of a chunk one physical block id, and the 2L plane
 // pointers one table.  The three arrays go to the device in one upload (a
-// pinned slot copied on a library stream that the caller's stream waits on),
-// then one launch per source class
+// pinned slot copied on a library stream that the caller's stream waits on), or,
+// where they are small, in the launches' own parameters; then one launch per source class
 // (per layer group, for layer-wise calls) moves the bytes:
 //   device-resident chunks  -> LDG or TMA kernel, HBM to HBM (on a library
 //                              stream joined back when host chunks run too);
@@ -450,13 +450,38 @@ int vec_bytes_for(uint64_t addr_or) {
 }
 
 // Copies the plan's tables into an upload slot and onto the device (caller stream).
+// Launches read these, or carry `host` in their parameters.
 struct Uploaded {
-    const Entry*    entries;
-    const int32_t*  blocks;
-    const int32_t*  blocks_cmp;
-    const uint64_t* planes;
-    UploadSlot*     slot;
+    const Entry*    entries = nullptr;
+    const int32_t*  blocks = nullptr;
+    const int32_t*  blocks_cmp = nullptr;
+    const uint64_t* planes = nullptr;
+    UploadSlot*     slot = nullptr;
+    const HostTables* host = nullptr;
 };
+
+HostTables host_tables(const Plan& pl) {
+    return {pl.planes.data(), pl.entries.data(), pl.blocks.data(),
+            (uint32_t)pl.planes.size(), (uint32_t)pl.entries.size(), (uint32_t)pl.blocks.size()};
+}
+
+// Whether a call's launches carry its tables.  An upload costs the call 3 to 4 us of
+// host time (a copy on another stream, three events, a wait) and the GPU a wait for
+// the copy, whatever its size; 3.5 KiB of parameters cost a launch 0.4 us.  So not
+// with more than kMostCarried launches.  Larger tables belong to calls of 100 us and
+// more, behind which the upload disappears.  A stream that is being captured takes
+// the upload, and fails as it does.
+constexpr int kMostCarried = 8;
+
+bool carry_tables(const HostTables& t, int launches, cudaStream_t s) {
+    if (launches > kMostCarried || !tables_fit(t)) return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return cs == cudaStreamCaptureStatusNone;
+}
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -519,7 +544,8 @@ Job make_job(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache, 
              const Uploaded& u, uint32_t first_entry, uint32_t num_entries, Mode mode,
              uint32_t plane_begin = 0, uint32_t plane_count = 0) {
     Job j{};
-    j.entries = u.entries + first_entry;
+    j.tables = u.host;
+    j.entries = u.entries ? u.entries + first_entry : nullptr;
     j.blocks = u.blocks;
     j.planes = u.planes;
     j.err = st.err;
@@ -778,9 +804,18 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     const Mode mode = retrieve ? MODE_RETRIEVE : MODE_STORE;
     const int host_grid = grid ? grid : f_few ? st.few_sm_ctas : (retrieve ? st.hostlink_ctas : st.store_ctas);
 
+    const HostTables tables = host_tables(pl);
     Uploaded u;
-    rc = upload(st, pl, s, u);
-    if (rc) return rc;
+    const bool plain_host = !pl.num_host || (host_variant == KVS_VARIANT_HOSTLINK && !f_few &&
+                                             !(flags & (KVS_F_PREFETCH_L2 | KVS_F_LAYER_SIGNAL)));
+    const bool plain_device = !pl.num_device || flavour != KVS_KERNEL_TMA || grid == 0;
+    if (plain_host && plain_device && !(flags & KVS_F_VALIDATE) &&
+        carry_tables(tables, groups * ((pl.num_host > 0) + (pl.num_device > 0)), s)) {
+        u.host = &tables;
+    } else {
+        rc = upload(st, pl, s, u);
+        if (rc) return rc;
+    }
     SlotGuard guard{u.slot, s};
     // Layer-wise, host chunks only: one persistent launch that publishes each
     // group's completion; the signal stream waits on the flags and records the
@@ -945,9 +980,17 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
     }
     pl.blocks_cmp.clear();
     cudaStream_t s = (cudaStream_t)stream;
+    const int L = g->num_layers;
+    const int lps = layers_per_step > 0 ? std::min(layers_per_step, L) : L;
+    const int groups = (L + lps - 1) / lps;
+    const HostTables tables = host_tables(pl);
     Uploaded u;
-    rc = upload(st, pl, s, u);
-    if (rc) return rc;
+    if (!few && !(flags & KVS_F_VALIDATE) && carry_tables(tables, groups * ((pl.num_host > 0) + (pl.num_device > 0)), s)) {
+        u.host = &tables;
+    } else {
+        rc = upload(st, pl, s, u);
+        if (rc) return rc;
+    }
     SlotGuard guard{u.slot, s};
     const int cap = (int)KVS_F_GET_MAX_CTAS(flags);
     const uint32_t hd = (uint32_t)(g->num_kv_heads * g->head_dim);
@@ -989,9 +1032,6 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
         ++g_launches;
         return KVS_OK;
     };
-    const int L = g->num_layers;
-    const int lps = layers_per_step > 0 ? std::min(layers_per_step, L) : L;
-    const int groups = (L + lps - 1) / lps;
     for (int k = 0; k < groups; ++k) {
         const uint32_t p0 = (uint32_t)(2 * k * lps);
         const uint32_t np = (uint32_t)(2 * (std::min(L, (k + 1) * lps) - k * lps));

@@ -41,6 +41,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "kvs.h"
 #include "kvs_async.cuh"
@@ -160,7 +161,7 @@ struct Fp8Span {
     uint64_t       codes;           // first code of the piece
     uint64_t       plane;           // base of the plane; long runs: plus the first code's offset in its run
     uint64_t       scales;          // H binary32 of the plane
-    const int32_t* blocks;          // physical block of the run that holds the first code, and on
+    uint32_t       run0;            // index of the block of the run that holds the first code
     uint32_t       off;             // short runs: offset of the first code in its run; long runs:
                                     // codes from it to the end of its run, at most piece_codes
     uint32_t       len;             // codes, a multiple of 16
@@ -168,7 +169,8 @@ struct Fp8Span {
 };
 
 // Piece q; false for pieces past the end of a short chunk.  Uniform across the CTA.
-__device__ __forceinline__ bool fp8_span(const Fp8Spans& dc, uint32_t q, Fp8Span& sp) {
+template <class TAB>
+__device__ __forceinline__ bool fp8_span(const Fp8Spans& dc, const TAB& tab, uint32_t q, Fp8Span& sp) {
     const Job& j = dc.f.job;
     const uint32_t ep = fdiv(q, dc.spp), k = q - ep * dc.spp.d, e = fdiv(ep, dc.planes);
     const uint32_t p = j.plane_begin + (ep - e * dc.planes.d);
@@ -181,7 +183,7 @@ __device__ __forceinline__ bool fp8_span(const Fp8Spans& dc, uint32_t q, Fp8Span
         i0 = fdiv((uint32_t)at, dc.run);
         row = fdiv((uint32_t)at / 16, dc.vpr);
     }
-    const Entry en = j.entries[e];
+    const Entry en = tab.entry(j.entry_base + e);
     const uint64_t span = (uint64_t)en.n_tok * (dc.f.heads * dc.f.head_dim);
     if (at >= span) return false;
     const uint64_t off = at - i0 * dc.run_codes;
@@ -189,8 +191,8 @@ __device__ __forceinline__ bool fp8_span(const Fp8Spans& dc, uint32_t q, Fp8Span
     sp.col = (uint32_t)(at / 16 - row * dc.vpr.d);
     sp.codes = en.chunk + dc.f.scale_bytes + (uint64_t)p * span + at;
     sp.scales = en.chunk + (uint64_t)p * dc.f.heads * 4;
-    sp.plane = j.planes[p] + (dc.long_runs ? off * 2 : 0);
-    sp.blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i0;
+    sp.plane = tab.plane(p) + (dc.long_runs ? off * 2 : 0);
+    sp.run0 = (j.entry_base + e) * j.blocks_per_chunk + (uint32_t)i0;
     sp.off = (uint32_t)(dc.long_runs ? min(dc.run_codes - off, (uint64_t)dc.piece_codes) : off);
     return true;
 }
@@ -239,8 +241,8 @@ struct RtRegs {
     int32_t blk[U];
 };
 
-template <int T, int U>
-__device__ __forceinline__ void rt_load(const Fp8Spans& dc, const Fp8Span& sp, RtRegs<U>& r) {
+template <int T, int U, class TAB>
+__device__ __forceinline__ void rt_load(const Fp8Spans& dc, const TAB& tab, const Fp8Span& sp, RtRegs<U>& r) {
     const uint32_t nv = sp.len / 16;
     bool bad = false;
 #pragma unroll
@@ -248,7 +250,7 @@ __device__ __forceinline__ void rt_load(const Fp8Spans& dc, const Fp8Span& sp, R
         const uint32_t v = threadIdx.x + u * T;
         if (v < nv) r.c[u] = ld_nc16(sp.codes + (uint64_t)v * 16);
         r.s[u] = __ldg(reinterpret_cast<const float*>(sp.scales) + fp8_vec_head(dc, sp, min(v, nv - 1)));
-        r.blk[u] = __ldg(sp.blocks + fp8_run(dc, sp, min(v, nv - 1) * 16));
+        r.blk[u] = tab.block(sp.run0 + fp8_run(dc, sp, min(v, nv - 1) * 16));
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
@@ -270,11 +272,12 @@ __device__ __forceinline__ void rt_store(const Fp8Spans& dc, const Fp8Span& sp, 
     }
 }
 
-__device__ __forceinline__ bool rt_next(const Fp8Spans& dc, uint32_t& q, Fp8Span& sp) {
+template <class TAB>
+__device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint32_t& q, Fp8Span& sp) {
     while (q < dc.num_pieces) {
         const uint32_t cur = q;
         q += gridDim.x;
-        if (fp8_span(dc, cur, sp)) return true;
+        if (fp8_span(dc, tab, cur, sp)) return true;
     }
     return false;
 }
@@ -284,30 +287,34 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, uint32_t& q, Fp8Span
 // that leaves them few SMs.  8192 tokens of the 8B shape: 2561 us with 128 threads x
 // 8 vectors and scales through shared memory, 2570 without it, 2555 here (the link:
 // 2541); 512 x 2 gains another 0.1% but fits two CTAs per SM.
-__global__ void __launch_bounds__(kRtLink, kRtLinkCtas) kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc) {
+template <bool INL>
+__global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
+kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
     RtRegs<kRtLinkVec> ra, rb;
     Fp8Span pa, pb;
     uint32_t q = blockIdx.x;
-    bool ha = rt_next(dc, q, pa);
-    if (ha) rt_load<kRtLink>(dc, pa, ra);
+    bool ha = rt_next(dc, tab, q, pa);
+    if (ha) rt_load<kRtLink>(dc, tab, pa, ra);
     while (ha) {
-        const bool hb = rt_next(dc, q, pb);
-        if (hb) rt_load<kRtLink>(dc, pb, rb);
+        const bool hb = rt_next(dc, tab, q, pb);
+        if (hb) rt_load<kRtLink>(dc, tab, pb, rb);
         rt_store<kRtLink>(dc, pa, ra);
         if (!hb) break;
-        ha = rt_next(dc, q, pa);
-        if (ha) rt_load<kRtLink>(dc, pa, ra);
+        ha = rt_next(dc, tab, q, pa);
+        if (ha) rt_load<kRtLink>(dc, tab, pa, ra);
         rt_store<kRtLink>(dc, pb, rb);
     }
 }
 
 // HBM chunks: one CTA per piece, no persistence; six CTAs per SM (four, or 128 threads x 8
 // vectors, or 512 x 2: up to 1% slower).
-__global__ void __launch_bounds__(kRtHbm, kRtHbmCtas) kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc) {
+template <bool INL>
+__global__ void __launch_bounds__(kRtHbm, kRtHbmCtas)
+kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
     Fp8Span sp;
-    if (!fp8_span(dc, blockIdx.x, sp)) return;              // uniform across the CTA
+    if (!fp8_span(dc, tab, blockIdx.x, sp)) return;              // uniform across the CTA
     RtRegs<kRtHbmVec> r;
-    rt_load<kRtHbm>(dc, sp, r);
+    rt_load<kRtHbm>(dc, tab, sp, r);
     rt_store<kRtHbm>(dc, sp, r);
 }
 
@@ -543,18 +550,18 @@ constexpr uint32_t kHeadMaxElems = kHeadVec * kStThreads * 8;
 // One segment of the store: FULL when every thread's kHeadVec vectors all lie in
 // the chunk (n * D/8 == kHeadVec * kStThreads, e.g. a 256-token chunk of head_dim
 // 128), so the loads and stores need no per-vector bounds test.
-template <bool FULL>
-__device__ __forceinline__ void store_head_segment(const Fp8Job& f, uint32_t e, uint32_t p, uint32_t h,
+template <bool FULL, class TAB>
+__device__ __forceinline__ void store_head_segment(const Fp8Job& f, const TAB& tab, uint32_t e, uint32_t p, uint32_t h,
                                                    uint32_t* warp_max, float* sm_inv) {
     const Job& j = f.job;
     const uint32_t H = f.heads, D = f.head_dim, vpt = D / 8;
     const uint32_t B = j.block_size, step = kStThreads / vpt;
     const uint32_t w = threadIdx.x % vpt, i0 = threadIdx.x / vpt;
     const uint64_t row2 = (uint64_t)H * D * 2;
-    const Entry en = j.entries[e];
+    const Entry en = tab.entry(j.entry_base + e);
     const uint32_t n = (uint32_t)en.n_tok;
-    const int32_t* blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk;
-    const uint64_t src0 = j.planes[p] + (uint64_t)h * D * 2 + (uint64_t)w * 16;
+    const uint32_t block0 = (j.entry_base + e) * j.blocks_per_chunk;
+    const uint64_t src0 = tab.plane(p) + (uint64_t)h * D * 2 + (uint64_t)w * 16;
     uint4 v[kHeadVec];
     uint32_t m2 = 0;
     bool bad = false;
@@ -564,7 +571,7 @@ __device__ __forceinline__ void store_head_segment(const Fp8Job& f, uint32_t e, 
         v[u] = make_uint4(0, 0, 0, 0);
         if (FULL || i < n) {
             const uint32_t bi = B == 1 ? i : __umulhi(i, f.block_magic), r = i - bi * B;
-            const int32_t blk = __ldg(blocks + bi);
+            const int32_t blk = tab.block(block0 + bi);
             if (blk < 0 || blk >= j.num_blocks) bad = true;
             else v[u] = ld_nc16(src0 + ((uint64_t)blk * B + r) * row2);
         }
@@ -597,7 +604,9 @@ __device__ __forceinline__ void store_head_segment(const Fp8Job& f, uint32_t e, 
     __syncthreads();                                       // warp_max / sm_inv are reused
 }
 
-__global__ void __launch_bounds__(kStThreads) kvs_fp8_store_head_kernel(const Fp8Job f, uint32_t num_segments) {
+template <bool INL>
+__global__ void __launch_bounds__(kStThreads)
+kvs_fp8_store_head_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t num_segments) {
     __shared__ uint32_t warp_max[kStThreads / 32];
     __shared__ float sm_inv;
     const Job& j = f.job;
@@ -606,10 +615,10 @@ __global__ void __launch_bounds__(kStThreads) kvs_fp8_store_head_kernel(const Fp
         const uint32_t eh = seg / H, h = seg - eh * H;
         const uint32_t e = eh / j.num_planes;
         const uint32_t p = j.plane_begin + (eh - e * j.num_planes);
-        if ((uint32_t)j.entries[e].n_tok == full_n)          // uniform across the CTA
-            store_head_segment<true>(f, e, p, h, warp_max, &sm_inv);
+        if ((uint32_t)tab.entry(j.entry_base + e).n_tok == full_n)          // uniform across the CTA
+            store_head_segment<true>(f, tab, e, p, h, warp_max, &sm_inv);
         else
-            store_head_segment<false>(f, e, p, h, warp_max, &sm_inv);
+            store_head_segment<false>(f, tab, e, p, h, warp_max, &sm_inv);
     }
 }
 
@@ -738,9 +747,9 @@ __device__ __forceinline__ void cluster_sync() {
 // Team k of T takes the units that begin in [k * W / T, (k + 1) * W / T) of the job's
 // W = sum over its chunks of (tokens + extra) x units per chunk.  CLUSTER: the tokens
 // of a unit are split over cl CTAs of a cluster, which exchange their maxima.
-template <int VEC, bool CLUSTER>
+template <int VEC, bool CLUSTER, bool INL>
 __global__ void __launch_bounds__(kUqThreads, uq_ctas(CLUSTER))
-kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t G, uint32_t extra, uint32_t cl) {
+kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t g, uint32_t G, uint32_t extra, uint32_t cl) {
     extern __shared__ __align__(128) uint8_t uq_smem[];
     uint32_t* rows = reinterpret_cast<uint32_t*>(uq_smem + uq_stage_bytes(VEC));   // plane row of each of the CTA's tokens
     // Maxima of unit n's heads in third n % 3, cleared before barrier n - 1: the readers of unit
@@ -751,7 +760,6 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
     __shared__ uint32_t all[CLUSTER ? 2 : 1][CLUSTER ? kUqMaxCluster : 1][kFp8MaxHeads];
     __shared__ uint32_t range[2];
     const Job& j = f.job;
-    const Entry* entries = j.entries;
     const uint32_t t = threadIdx.x, D = f.head_dim, vph = D / 8, vpt = g * vph, step = kUqThreads / vpt;
     const uint32_t w = t % vpt, i0 = t / vpt, hl = w / vph;
     const uint32_t peers = __match_any_sync(0xFFFFFFFFu, i0 < step ? hl : 0xFFFFu);   // lanes on the same head
@@ -764,8 +772,9 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
         const uint64_t W = (f.tokens + (uint64_t)extra * j.num_entries) * upe;
         const uint64_t x[2] = {W * team / teams, W * (team + 1) / teams};
         for (uint32_t e = t; e < j.num_entries; e += kUqThreads) {
-            const uint64_t at = (entries[e].first_tok + (uint64_t)extra * e) * upe;
-            const uint32_t n = (uint32_t)entries[e].n_tok + extra;
+            const Entry en = tab.entry(j.entry_base + e);
+            const uint64_t at = (en.first_tok + (uint64_t)extra * e) * upe;
+            const uint32_t n = (uint32_t)en.n_tok + extra;
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 if (x[k] >= at && x[k] < at + (uint64_t)n * upe) range[k] = (uint32_t)((uint64_t)e * upe + (x[k] - at + n - 1) / n);
@@ -782,14 +791,14 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
     uint32_t mine = 0, first = 0;                           // the CTA's tokens of the chunk (0 for an idle thread), from `first`
     // the chunk's plane rows; a block out of range, which the planner has excluded, is reported
     auto enter = [&]() {
-        const uint32_t n = (uint32_t)entries[c.e].n_tok, B = j.block_size;
-        const int32_t* blocks = j.blocks + (size_t)(j.entry_base + c.e) * j.blocks_per_chunk;
+        const uint32_t n = (uint32_t)tab.entry(j.entry_base + c.e).n_tok, B = j.block_size;
+        const uint32_t block0 = (j.entry_base + c.e) * j.blocks_per_chunk;
         const uint32_t per = CLUSTER ? (n + cl - 1) / cl : n;
         first = CLUSTER ? min(rank * per, n) : 0;
         const uint32_t count = min(per, n - first);
         for (uint32_t r = t; r < count; r += kUqThreads) {
             const uint32_t i = first + r, bi = B == 1 ? i : __umulhi(i, f.block_magic);
-            uint32_t blk = (uint32_t)__ldg(blocks + bi);
+            uint32_t blk = (uint32_t)tab.block(block0 + bi);
             if (blk >= (uint32_t)j.num_blocks) {
                 atomicCAS(j.err, 0, KVS_ERR_BOUNDS);
                 blk = 0;
@@ -800,7 +809,7 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
         __syncthreads();
     };
     const uint32_t row2 = f.heads * D * 2;
-    auto source = [&]() { return j.planes[c.p] + (uint64_t)(c.group * vpt + w) * 16; };
+    auto source = [&]() { return tab.plane(c.p) + (uint64_t)(c.group * vpt + w) * 16; };
     enter();
     const uint32_t slot0 = smem_u32(uq_smem) + t * 16;      // this thread's vector u at slot0 + u * kUqThreads * 16
     {
@@ -859,7 +868,7 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
         }
         const float af = __uint_as_float(a << 16);
         const float inv = af > 0.0f ? __fdiv_rn(448.0f, af) : 1.0f;
-        const Entry en = entries[c.e];
+        const Entry en = tab.entry(j.entry_base + c.e);
         const uint32_t h0 = c.group * g, hd = f.heads * D, old = mine;
         if (rank == 0 && i0 == 0 && w % vph == 0)
             reinterpret_cast<float*>(en.chunk)[(uint64_t)c.p * f.heads + h0 + hl] = af > 0.0f ? __fdiv_rn(af, 448.0f) : 1.0f;
@@ -889,7 +898,9 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, uint32_t g, uint32_t
 constexpr int kStUnroll = 4;                         // vectors per thread in flight per step
 
 // One CTA per (entry, plane) segment: the chunk's n tokens of that plane.
-__global__ void __launch_bounds__(kStThreads) kvs_fp8_store_kernel(const Fp8Job f, uint32_t num_segments) {
+template <bool INL>
+__global__ void __launch_bounds__(kStThreads)
+kvs_fp8_store_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t num_segments) {
     __shared__ uint32_t amax[kFp8MaxHeads];
     __shared__ float scale[kFp8MaxHeads];                    // holds 448 / amax per head
     const Job& j = f.job;
@@ -898,17 +909,17 @@ __global__ void __launch_bounds__(kStThreads) kvs_fp8_store_kernel(const Fp8Job 
     for (uint32_t seg = blockIdx.x; seg < num_segments; seg += gridDim.x) {
         const uint32_t e = seg / j.num_planes;
         const uint32_t p = j.plane_begin + (seg - e * j.num_planes);
-        const Entry en = j.entries[e];
+        const Entry en = tab.entry(j.entry_base + e);
         const uint32_t n = (uint32_t)en.n_tok;
-        const int32_t* blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk;
-        const uint64_t plane = j.planes[p];
+        const uint32_t block0 = (j.entry_base + e) * j.blocks_per_chunk;
+        const uint64_t plane = tab.plane(p);
         const uint64_t codes = en.chunk + f.scale_bytes + (uint64_t)p * n * vpr * 16;
         const uint32_t nvec = n * vpr;
         // source address of vector v (16 BF16 = 32 bytes), or 0 for a bad block
         auto src_of = [&](uint32_t v, uint32_t& h) -> uint64_t {
             const uint32_t i = v / vpr, w = v - i * vpr;
             h = w / vph;
-            const int32_t blk = __ldg(blocks + i / j.block_size);
+            const int32_t blk = tab.block(block0 + i / j.block_size);
             if (blk < 0 || blk >= j.num_blocks) return 0;
             return plane + ((uint64_t)blk * j.block_size + i % j.block_size) * row2 + (uint64_t)w * 32;
         };
@@ -1032,9 +1043,11 @@ cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s) {
     while (piece > kFp8PieceCodes / 4 && total / piece < 2ull * (per_piece ? sm_count() : grid)) piece /= 2;
     const Fp8Spans dc = make_spans(fj, piece);
     const uint32_t ctas = per_piece ? dc.num_pieces : std::min<uint32_t>((uint32_t)grid, dc.num_pieces);
-    if (per_piece) kvs_fp8_retrieve_piece_kernel<<<ctas, kRtHbm, 0, s>>>(dc);
-    else kvs_fp8_retrieve_kernel<<<ctas, kRtLink, 0, s>>>(dc);
-    return cudaGetLastError();
+    return with_tables(fj.job, [&](const auto& tab) {
+        constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+        if (per_piece) kvs_fp8_retrieve_piece_kernel<I><<<ctas, kRtHbm, 0, s>>>(dc, tab);
+        else kvs_fp8_retrieve_kernel<I><<<ctas, kRtLink, 0, s>>>(dc, tab);
+    });
 }
 
 cudaError_t launch_fp8_retrieve_staged(const Fp8Job& fj, int grid, cudaStream_t s) {
@@ -1076,13 +1089,14 @@ uint32_t uq_heads(const Fp8Job& fj, uint32_t chunk_tokens, uint32_t vec) {
     return 0;
 }
 
-template <int VEC, bool CLUSTER>
-cudaError_t launch_unit(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chunk_tokens, uint32_t g, uint32_t cl) {
+template <int VEC, bool CLUSTER, bool INL>
+cudaError_t launch_unit(const Fp8Job& fj, const Tables<INL>& tab, int grid, cudaStream_t s, uint32_t chunk_tokens, uint32_t g,
+                        uint32_t cl) {
     if (fj.job.num_entries == 0) return cudaSuccess;
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= kMaxDev) dev = 0;
-    const auto k = kvs_fp8_store_unit_kernel<VEC, CLUSTER>;
+    const auto k = kvs_fp8_store_unit_kernel<VEC, CLUSTER, INL>;
     static bool attr[kMaxDev];                              // shared-memory limit raised
     if (!attr[dev]) {
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1119,7 +1133,7 @@ cudaError_t launch_unit(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chu
     const uint32_t G = uq_team(fj.heads / g, (uint32_t)ctas);
     cfg.gridDim = dim3((uint32_t)ctas / G * G * cl);
     const uint32_t extra = kUqUnitBytes / (g * fj.head_dim * 2);
-    return cudaLaunchKernelEx(&cfg, k, fj, g, G, extra, cl);
+    return cudaLaunchKernelEx(&cfg, k, fj, tab, g, G, extra, cl);
 }
 
 cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_t chunk_tokens, bool staged) {
@@ -1128,26 +1142,38 @@ cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_
     // sizes below 2^16), a row table of at most 16 KiB.
     if (staged && chunk_tokens <= kUqMaxRows && (uint64_t)fj.job.num_blocks * fj.job.block_size <= 0xFFFFFFFFull) {
         const uint32_t g = uq_heads(fj, chunk_tokens, kUqVec), gw = uq_heads(fj, chunk_tokens, kUqVecWide);
-        if (gw > g) return launch_unit<kUqVecWide, false>(fj, grid, s, chunk_tokens, gw, 1);
-        if (g) return launch_unit<kUqVec, false>(fj, grid, s, chunk_tokens, g, 1);
-        uint32_t cl = 2;
-        while (cl <= kUqMaxCluster && vpt <= kUqThreads && kUqVec * (kUqThreads / vpt) * cl < chunk_tokens) cl *= 2;
-        if (cl <= kUqMaxCluster && vpt <= kUqThreads && (grid <= 0 || grid >= (int)cl))
-            return launch_unit<kUqVec, true>(fj, grid, s, chunk_tokens, 1, cl);
+        uint32_t cl = 1;
+        if (!g && !gw) {
+            cl = 2;
+            while (cl <= kUqMaxCluster && vpt <= kUqThreads && kUqVec * (kUqThreads / vpt) * cl < chunk_tokens) cl *= 2;
+        }
+        if (cl <= kUqMaxCluster && vpt <= kUqThreads && (grid <= 0 || grid >= (int)cl)) {
+            cudaError_t e = cudaSuccess;
+            const cudaError_t last = with_tables(fj.job, [&](const auto& tab) {
+                e = cl > 1   ? launch_unit<kUqVec, true>(fj, tab, grid, s, chunk_tokens, 1, cl)
+                    : gw > g ? launch_unit<kUqVecWide, false>(fj, tab, grid, s, chunk_tokens, gw, 1)
+                             : launch_unit<kUqVec, false>(fj, tab, grid, s, chunk_tokens, g, 1);
+            });
+            return e != cudaSuccess ? e : last;
+        }
     }
     if ((uint64_t)chunk_tokens * fj.head_dim <= kHeadMaxElems && kStThreads % vpt == 0 && chunk_tokens < 65536 &&
         fj.job.block_size < 65536) {
         const uint64_t segs = (uint64_t)fj.job.num_entries * fj.job.num_planes * fj.heads;
         if (segs == 0) return cudaSuccess;
         if (grid <= 0 || (uint64_t)grid > segs) grid = (int)std::min<uint64_t>(segs, 1u << 30);
-        kvs_fp8_store_head_kernel<<<grid, kStThreads, 0, s>>>(fj, (uint32_t)segs);
-        return cudaGetLastError();
+        return with_tables(fj.job, [&](const auto& tab) {
+            constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+            kvs_fp8_store_head_kernel<I><<<grid, kStThreads, 0, s>>>(fj, tab, (uint32_t)segs);
+        });
     }
     const uint64_t segs = (uint64_t)fj.job.num_entries * fj.job.num_planes;
     if (segs == 0) return cudaSuccess;
     if (grid <= 0 || (uint64_t)grid > segs) grid = (int)segs;
-    kvs_fp8_store_kernel<<<grid, kStThreads, 0, s>>>(fj, (uint32_t)segs);
-    return cudaGetLastError();
+    return with_tables(fj.job, [&](const auto& tab) {
+        constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+        kvs_fp8_store_kernel<I><<<grid, kStThreads, 0, s>>>(fj, tab, (uint32_t)segs);
+    });
 }
 
 }  // namespace kvs

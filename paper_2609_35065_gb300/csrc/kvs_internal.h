@@ -23,6 +23,21 @@ enum Mode : int32_t {
     MODE_COMPARE  = 2,  // flag KVS_ERR_ALIAS where chunk bytes differ from plane bytes
 };
 
+// A call's tables on the host, where a launch carries them in its parameters.
+struct HostTables {
+    const uint64_t* planes;
+    const Entry*    entries;         // of all classes
+    const int32_t*  blocks;
+    uint32_t num_planes, num_entries, num_blocks;
+};
+
+// What a launch can carry: with its other parameters within 4 KiB.
+constexpr uint32_t kTableBytes = 3584;
+
+inline bool tables_fit(const HostTables& t) {
+    return (uint64_t)t.num_planes * 8 + (uint64_t)t.num_entries * sizeof(Entry) + (uint64_t)t.num_blocks * 4 + 8 <= kTableBytes;
+}
+
 // Work of one launch.  A "run" is the contiguous copy of one (entry, plane p,
 // block i of the chunk): up to B token rows, B*R bytes, contiguous on both
 // sides.  Runs are cut into "pieces" of at most piece_bytes for the kernels.
@@ -45,6 +60,7 @@ struct Job {
     uint32_t        piece_bytes;     // multiple of 16
     uint32_t        block_size;      // B
     int32_t         mode;            // Mode
+    const HostTables* tables;        // not null: entries, blocks and planes are not uploaded
     uint32_t        align;           // OR of the plane and chunk addresses and of every n_tok * R (low bits)
 };
 

@@ -2,6 +2,9 @@
 #pragma once
 
 #include <cstdint>
+#include <cstring>
+
+#include "kvs_internal.h"
 
 namespace kvs {
 namespace {
@@ -28,6 +31,53 @@ inline FastDiv make_fastdiv(uint32_t d) {
 
 __device__ __forceinline__ uint32_t fdiv(uint32_t n, const FastDiv& f) {
     return (uint32_t)(((uint64_t)n * f.m) >> f.p);
+}
+
+// ---------------------------------------------------------------------------
+// How a kernel reads the call's tables: from device memory, where the planner has
+// uploaded them, or from its own parameters.  A small call spends most of its time
+// on the upload (a copy on another stream, two events, a wait); tables that fit are
+// passed by value instead.
+// ---------------------------------------------------------------------------
+template <bool INL>
+struct Tables;
+
+template <>
+struct Tables<false> {
+    static constexpr bool kInline = false;
+    const Entry*    entries;             // entry_base entries before the job's first
+    const int32_t*  blocks;
+    const uint64_t* planes;
+    __host__ __device__ explicit Tables(const Job& j)
+        : entries(j.entries - j.entry_base), blocks(j.blocks), planes(j.planes) {}
+    __device__ __forceinline__ Entry entry(uint32_t e) const { return entries[e]; }
+    __device__ __forceinline__ int32_t block(uint32_t k) const { return __ldg(blocks + k); }
+    __device__ __forceinline__ uint64_t plane(uint32_t p) const { return planes[p]; }
+};
+
+template <>
+struct Tables<true> {
+    static constexpr bool kInline = true;
+    uint32_t entries_at, blocks_at;
+    alignas(16) unsigned char raw[kTableBytes];
+    explicit Tables(const HostTables& t) {
+        entries_at = (t.num_planes * 8 + 15) / 16 * 16;
+        blocks_at = entries_at + t.num_entries * (uint32_t)sizeof(Entry);
+        memcpy(raw, t.planes, t.num_planes * 8);
+        memcpy(raw + entries_at, t.entries, t.num_entries * sizeof(Entry));
+        memcpy(raw + blocks_at, t.blocks, t.num_blocks * 4);
+    }
+    __device__ __forceinline__ Entry entry(uint32_t e) const { return reinterpret_cast<const Entry*>(raw + entries_at)[e]; }
+    __device__ __forceinline__ int32_t block(uint32_t k) const { return reinterpret_cast<const int32_t*>(raw + blocks_at)[k]; }
+    __device__ __forceinline__ uint64_t plane(uint32_t p) const { return reinterpret_cast<const uint64_t*>(raw)[p]; }
+};
+
+// launch(tables) with the tables of `job`, by value or by pointer.
+template <class F>
+cudaError_t with_tables(const Job& job, F&& launch) {
+    if (job.tables) launch(Tables<true>(*job.tables));
+    else launch(Tables<false>(job));
+    return cudaGetLastError();
 }
 
 }  // namespace

@@ -23,6 +23,7 @@
 //    of hanging.
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "kvs.h"
 #include "kvs_async.cuh"
@@ -45,7 +46,8 @@ struct Piece {
 
 // Piece q -> addresses.  Returns false for pieces with nothing to move
 // (past the end of a short chunk, a skipped block, a bounds violation).
-__device__ __forceinline__ bool decode_piece(const Decoder& dc, uint32_t q, Piece& pc) {
+template <class T>
+__device__ __forceinline__ bool decode_piece(const Decoder& dc, const T& tab, uint32_t q, Piece& pc) {
     const Job& j = dc.job;
     const uint32_t g = fdiv(q, dc.ppr);
     const uint32_t k = q - g * dc.ppr.d;
@@ -54,8 +56,8 @@ __device__ __forceinline__ bool decode_piece(const Decoder& dc, uint32_t q, Piec
     const uint32_t e = fdiv(ep, dc.planes);
     const uint32_t p = j.plane_begin + (ep - e * dc.planes.d);
     // The two descriptor loads are independent, so both are in flight at once.
-    const int32_t blk = __ldg(j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i);
-    const Entry en = j.entries[e];
+    const int32_t blk = tab.block((j.entry_base + e) * j.blocks_per_chunk + i);
+    const Entry en = tab.entry(j.entry_base + e);
     const int64_t first = (int64_t)i * j.block_size;
     const int64_t ntok = min((int64_t)j.block_size, (int64_t)en.n_tok - first);
     if (ntok <= 0) return false;
@@ -69,8 +71,12 @@ __device__ __forceinline__ bool decode_piece(const Decoder& dc, uint32_t q, Piec
     if (off >= run_bytes) return false;
     pc.len = (uint32_t)min((uint64_t)j.piece_bytes, run_bytes - off);
     pc.chunk_addr = en.chunk + ((uint64_t)p * (uint64_t)en.n_tok + (uint64_t)first) * j.row_bytes + off;
-    pc.plane_addr = j.planes[p] + (uint64_t)blk * j.block_size * j.row_bytes + off;
+    pc.plane_addr = tab.plane(p) + (uint64_t)blk * j.block_size * j.row_bytes + off;
     return true;
+}
+
+__device__ __forceinline__ bool decode_piece(const Decoder& dc, uint32_t q, Piece& pc) {
+    return decode_piece(dc, Tables<false>(dc.job), q, pc);
 }
 
 // ---------------------------------------------------------------------------
@@ -191,14 +197,15 @@ struct SpanDecoder {
 struct SpanPiece {
     uint64_t       chunk;  // address of the piece's first byte in the chunk
     uint64_t       plane;  // base of its plane; long runs: plus the first byte's offset in its run
-    const int32_t* blocks; // physical block of the run that holds the first byte, and on
+    uint32_t       run0;   // index of the block of the run that holds the first byte
     uint32_t       off;    // short runs: offset of the first byte in its run; long runs: bytes
                            // from it to the end of its run, at most piece_bytes
     uint32_t       len;
 };
 
 // Piece q; false for pieces past the end of a short chunk.  Uniform across the CTA.
-__device__ __forceinline__ bool span_piece(const SpanDecoder& dc, uint32_t q, SpanPiece& sp) {
+template <class T>
+__device__ __forceinline__ bool span_piece(const SpanDecoder& dc, const T& tab, uint32_t q, SpanPiece& sp) {
     const Job& j = dc.job;
     const uint32_t ep = fdiv(q, dc.spp);
     const uint32_t k = q - ep * dc.spp.d;
@@ -208,14 +215,14 @@ __device__ __forceinline__ bool span_piece(const SpanDecoder& dc, uint32_t q, Sp
     uint64_t i0;
     if (dc.far_spans) i0 = at / dc.run_bytes;
     else i0 = fdiv((uint32_t)at, dc.run);
-    const Entry en = j.entries[e];
+    const Entry en = tab.entry(j.entry_base + e);
     const uint64_t span = (uint64_t)en.n_tok * j.row_bytes;
     if (at >= span) return false;
     sp.len = (uint32_t)min((uint64_t)j.piece_bytes, span - at);
     const uint64_t off = at - i0 * dc.run_bytes;
     sp.chunk = en.chunk + (uint64_t)p * span + at;
-    sp.plane = j.planes[p] + (dc.long_runs ? off : 0);
-    sp.blocks = j.blocks + (size_t)(j.entry_base + e) * j.blocks_per_chunk + i0;
+    sp.plane = tab.plane(p) + (dc.long_runs ? off : 0);
+    sp.run0 = (j.entry_base + e) * j.blocks_per_chunk + (uint32_t)i0;
     sp.off = (uint32_t)(dc.long_runs ? min(dc.run_bytes - off, (uint64_t)j.piece_bytes) : off);
     return true;
 }
@@ -237,13 +244,13 @@ __device__ __forceinline__ uint64_t span_plane(const SpanDecoder& dc, const Span
 // writes, or one out of range, which the planner has excluded).  A retrieval looks
 // all its blocks up first, without a branch between them; a store-back, whose loads
 // need the blocks, issues each load as soon as its own lookup is back.
-template <int MODE, int V, int U>
-__device__ __forceinline__ void span_load(const SpanDecoder& dc, const SpanPiece& sp, uint32_t base, uint32_t T,
-                                          uint32_t n, int32_t (&blk)[U], typename Vec<V>::T (&r)[U]) {
+template <int MODE, int V, int U, class TAB>
+__device__ __forceinline__ void span_load(const SpanDecoder& dc, const TAB& tab, const SpanPiece& sp, uint32_t base,
+                                          uint32_t T, uint32_t n, int32_t (&blk)[U], typename Vec<V>::T (&r)[U]) {
     bool bad = false;
     auto look = [&](int u) {
         const uint32_t k = base + u * T;
-        blk[u] = __ldg(sp.blocks + span_run(dc, sp, min(k, n - 1) * V));
+        blk[u] = tab.block(sp.run0 + span_run(dc, sp, min(k, n - 1) * V));
         const bool in = (uint32_t)blk[u] < (uint32_t)dc.job.num_blocks;
         bad |= !in && blk[u] >= 0;
         if (!in || k >= n) blk[u] = -1;
@@ -285,28 +292,28 @@ __device__ __forceinline__ bool span_wide(const SpanDecoder& dc, const SpanPiece
 }
 
 // The rest of a span that is no multiple of 16 bytes: at most 15 bytes of one run.
-template <int MODE>
-__device__ __forceinline__ void span_tail(const SpanDecoder& dc, const SpanPiece& sp) {
+template <int MODE, class TAB>
+__device__ __forceinline__ void span_tail(const SpanDecoder& dc, const TAB& tab, const SpanPiece& sp) {
     const uint32_t x = (sp.len & ~15u) + threadIdx.x;
     if (x >= sp.len) return;
     uint8_t r[1];
     int32_t blk[1];
-    span_load<MODE, 1, 1>(dc, sp, x, 0, sp.len, blk, r);
+    span_load<MODE, 1, 1>(dc, tab, sp, x, 0, sp.len, blk, r);
     span_store<MODE, 1, 1>(dc, sp, x, 0, blk, r);
 }
 
 // A piece whose two sides do not share 16-byte alignment (the last chunk of a
 // request where n * R is no multiple of 16, runs that are none): vectors of V, run
 // by run where a run has work for every thread.
-template <int MODE, int V, int U>
-__device__ __forceinline__ void span_narrow(const SpanDecoder& dc, const SpanPiece& sp) {
+template <int MODE, int V, int U, class TAB>
+__device__ __forceinline__ void span_narrow(const SpanDecoder& dc, const TAB& tab, const SpanPiece& sp) {
     using T = typename Vec<V>::T;
     if (dc.run_bytes >= blockDim.x * V) {
         uint32_t end;
         for (uint32_t x = 0; x < sp.len; x = end) {      // uniform across the CTA
             const uint32_t i = span_run(dc, sp, x);
             end = min(sp.len, dc.long_runs ? (i ? sp.len : sp.off) : (i + 1) * (uint32_t)dc.run_bytes - sp.off);
-            const int32_t blk = __ldg(sp.blocks + i);
+            const int32_t blk = tab.block(sp.run0 + i);
             if (blk < 0) continue;
             if (blk >= dc.job.num_blocks) {
                 atomicCAS(dc.job.err, 0, KVS_ERR_BOUNDS);
@@ -332,7 +339,7 @@ __device__ __forceinline__ void span_narrow(const SpanDecoder& dc, const SpanPie
     for (uint32_t base = threadIdx.x; base < n; base += blockDim.x * U) {
         T r[U];
         int32_t blk[U];
-        span_load<MODE, V, U>(dc, sp, base, blockDim.x, n, blk, r);
+        span_load<MODE, V, U>(dc, tab, sp, base, blockDim.x, n, blk, r);
         span_store<MODE, V, U>(dc, sp, base, blockDim.x, blk, r);
     }
 }
@@ -346,33 +353,34 @@ constexpr int kSpanThreads = 512;
 constexpr int kSpanCtasPerSm = 4;
 constexpr int kSpanUnroll = kPieceBytes / 16 / kSpanThreads;
 
-template <int MODE, bool TAIL>
+template <int MODE, bool TAIL, bool INL>
 __global__ void __launch_bounds__(kSpanThreads, TAIL ? 3 : kSpanCtasPerSm)
-kvs_span_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+kvs_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
-        if (!span_piece(dc, q, sp)) continue;            // uniform across the CTA
+        if (!span_piece(dc, tab, q, sp)) continue;            // uniform across the CTA
         if (TAIL && !span_wide(dc, sp)) continue;
         uint4 r[kSpanUnroll];
         int32_t blk[kSpanUnroll];
-        span_load<MODE, 16, kSpanUnroll>(dc, sp, threadIdx.x, kSpanThreads, sp.len / 16, blk, r);
+        span_load<MODE, 16, kSpanUnroll>(dc, tab, sp, threadIdx.x, kSpanThreads, sp.len / 16, blk, r);
         span_store<MODE, 16, kSpanUnroll>(dc, sp, threadIdx.x, kSpanThreads, blk, r);
-        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, sp);
+        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, tab, sp);
     }
 }
 
 // The other pieces, in a kernel of its own: as a branch of the one above, its
 // registers spill there or halve its CTAs (aligned 120-byte rows: 9.4 -> 13 us).
-template <int MODE>
-__global__ void __launch_bounds__(kSpanThreads, 3) kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+template <int MODE, bool INL>
+__global__ void __launch_bounds__(kSpanThreads, 3)
+kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
-        if (!span_piece(dc, q, sp) || span_wide(dc, sp)) continue;   // uniform across the CTA
+        if (!span_piece(dc, tab, q, sp) || span_wide(dc, sp)) continue;   // uniform across the CTA
         const uint32_t a = (uint32_t)sp.chunk | (uint32_t)sp.plane | sp.off | (uint32_t)dc.run_bytes | sp.len;
-        if ((a & 7) == 0) span_narrow<MODE, 8, 4>(dc, sp);
-        else if ((a & 3) == 0) span_narrow<MODE, 4, 4>(dc, sp);
-        else if ((a & 1) == 0) span_narrow<MODE, 2, 4>(dc, sp);
-        else span_narrow<MODE, 1, 4>(dc, sp);
+        if ((a & 7) == 0) span_narrow<MODE, 8, 4>(dc, tab, sp);
+        else if ((a & 3) == 0) span_narrow<MODE, 4, 4>(dc, tab, sp);
+        else if ((a & 1) == 0) span_narrow<MODE, 2, 4>(dc, tab, sp);
+        else span_narrow<MODE, 1, 4>(dc, tab, sp);
     }
 }
 
@@ -383,11 +391,12 @@ __global__ void __launch_bounds__(kSpanThreads, 3) kvs_span_narrow_kernel(const 
 constexpr int kPieceThreads = 512;
 constexpr int kPieceUnroll = kPieceBytes / 16 / kPieceThreads;
 
-template <int MODE>
-__global__ void __launch_bounds__(kPieceThreads, 4) kvs_ldg_piece_kernel(const Decoder dc) {
+template <int MODE, bool INL>
+__global__ void __launch_bounds__(kPieceThreads, 4)
+kvs_ldg_piece_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab) {
     static_assert(kPieceUnroll * kPieceThreads * 16 == kPieceBytes, "one piece per CTA");
     Piece pc;
-    if (!decode_piece(dc, blockIdx.x, pc)) return;       // uniform across the CTA
+    if (!decode_piece(dc, tab, blockIdx.x, pc)) return;  // uniform across the CTA
     const uint4* s = reinterpret_cast<const uint4*>(MODE == MODE_RETRIEVE ? pc.chunk_addr : pc.plane_addr);
     uint4* d = reinterpret_cast<uint4*>(MODE == MODE_RETRIEVE ? pc.plane_addr : pc.chunk_addr);
     const uint32_t n = pc.len / 16;
@@ -415,11 +424,12 @@ __global__ void __launch_bounds__(kPieceThreads, 4) kvs_ldg_piece_kernel(const D
 // registers, so the loads of the next piece are in flight while the current
 // one is stored.  A CTA then always has 32-64 KiB outstanding over the
 // long-latency host link, and a small grid saturates it.
-__device__ __forceinline__ bool next_piece_ldg(const Decoder& dc, uint32_t num_pieces, uint32_t& q, Piece& pc) {
+template <class T>
+__device__ __forceinline__ bool next_piece_ldg(const Decoder& dc, const T& tab, uint32_t num_pieces, uint32_t& q, Piece& pc) {
     while (q < num_pieces) {
         const uint32_t cur = q;
         q += gridDim.x;
-        if (decode_piece(dc, cur, pc)) return true;
+        if (decode_piece(dc, tab, cur, pc)) return true;
     }
     return false;
 }
@@ -444,21 +454,22 @@ __device__ __forceinline__ void store_piece16(uint64_t dst, uint32_t len, const 
     }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(kLdgThreads) kvs_link_kernel(const Decoder dc, uint32_t num_pieces) {
+template <int MODE, bool INL>
+__global__ void __launch_bounds__(kLdgThreads)
+kvs_link_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
     static_assert(kPieceBytes == kLdgUnroll * kLdgThreads * 16, "one piece per register set");
     constexpr bool to_plane = (MODE == MODE_RETRIEVE);
     uint4 ra[kLdgUnroll], rb[kLdgUnroll];
     Piece pa, pb;
     uint32_t q = blockIdx.x;
-    bool ha = next_piece_ldg(dc, num_pieces, q, pa);
+    bool ha = next_piece_ldg(dc, tab, num_pieces, q, pa);
     if (ha) load_piece16(to_plane ? pa.chunk_addr : pa.plane_addr, pa.len, ra);
     while (ha) {
-        const bool hb = next_piece_ldg(dc, num_pieces, q, pb);
+        const bool hb = next_piece_ldg(dc, tab, num_pieces, q, pb);
         if (hb) load_piece16(to_plane ? pb.chunk_addr : pb.plane_addr, pb.len, rb);
         store_piece16(to_plane ? pa.plane_addr : pa.chunk_addr, pa.len, ra);
         if (!hb) break;
-        ha = next_piece_ldg(dc, num_pieces, q, pa);
+        ha = next_piece_ldg(dc, tab, num_pieces, q, pa);
         if (ha) load_piece16(to_plane ? pa.chunk_addr : pa.plane_addr, pa.len, ra);
         store_piece16(to_plane ? pb.plane_addr : pb.chunk_addr, pb.len, rb);
     }
@@ -468,8 +479,9 @@ __global__ void __launch_bounds__(kLdgThreads) kvs_link_kernel(const Decoder dc,
 // run alone gives a 256-thread CTA run_bytes / 4096 vectors a thread, and the link
 // wants megabytes in flight: with 2 KiB runs, retrieval 340 -> 239 us and
 // store-back 279 -> 269 us at 49 MB (the link's own time: 233 and 254).
-template <int MODE, bool TAIL>
-__global__ void __launch_bounds__(kLdgThreads, 2) kvs_link_span_kernel(const __grid_constant__ SpanDecoder dc, uint32_t num_pieces) {
+template <int MODE, bool TAIL, bool INL>
+__global__ void __launch_bounds__(kLdgThreads, 2)
+kvs_link_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
     uint4 ra[kLdgUnroll], rb[kLdgUnroll];
     int32_t ba[kLdgUnroll], bb[kLdgUnroll];
     SpanPiece pa, pb;
@@ -478,16 +490,16 @@ __global__ void __launch_bounds__(kLdgThreads, 2) kvs_link_span_kernel(const __g
         while (q < num_pieces) {
             const uint32_t cur = q;
             q += gridDim.x;
-            if (span_piece(dc, cur, sp) && (!TAIL || span_wide(dc, sp))) return true;
+            if (span_piece(dc, tab, cur, sp) && (!TAIL || span_wide(dc, sp))) return true;
         }
         return false;
     };
     auto load = [&](const SpanPiece& sp, int32_t (&blk)[kLdgUnroll], uint4 (&r)[kLdgUnroll]) {
-        span_load<MODE, 16, kLdgUnroll>(dc, sp, threadIdx.x, kLdgThreads, sp.len / 16, blk, r);
+        span_load<MODE, 16, kLdgUnroll>(dc, tab, sp, threadIdx.x, kLdgThreads, sp.len / 16, blk, r);
     };
     auto store = [&](const SpanPiece& sp, const int32_t (&blk)[kLdgUnroll], const uint4 (&r)[kLdgUnroll]) {
         span_store<MODE, 16, kLdgUnroll>(dc, sp, threadIdx.x, kLdgThreads, blk, r);
-        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, sp);
+        if (TAIL && (sp.len & 15)) span_tail<MODE>(dc, tab, sp);
     };
     bool ha = next(pa);
     if (ha) load(pa, ba, ra);
@@ -564,7 +576,7 @@ __global__ void __launch_bounds__(kLdgThreads, 2) kvs_link_staged_kernel(const D
     // fill slot s with the CTA's next piece; a shared-memory slot always commits
     // one group (empty past the end), so wait_group counts pieces
     auto fill = [&](int s) {
-        has[s] = next_piece_ldg(dc, num_pieces, q, pc[s]);
+        has[s] = next_piece_ldg(dc, Tables<false>(dc.job), num_pieces, q, pc[s]);
         if (s == 0) {
             if (has[s]) load_piece16(pc[s].chunk_addr, pc[s].len, r);
         } else {
@@ -809,13 +821,14 @@ __global__ void __launch_bounds__(32, 1) kvs_tma_kernel(const Decoder dc, uint32
 // (completing on an mbarrier, bounded wait) and one bulk store, and leaves once
 // the store has read the stage.  Shared memory allows six such CTAs per SM,
 // 192 KiB of loads in flight, with almost no registers.
-template <int MODE>
-__global__ void __launch_bounds__(32) kvs_tma_piece_kernel(const Decoder dc) {
+template <int MODE, bool INL>
+__global__ void __launch_bounds__(32)
+kvs_tma_piece_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab) {
     extern __shared__ __align__(128) uint8_t stage[];
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x != 0) return;
     Piece pc;
-    if (!decode_piece(dc, blockIdx.x, pc)) return;
+    if (!decode_piece(dc, tab, blockIdx.x, pc)) return;
     const uint32_t b = smem_u32(&bar);
     mbar_init(b, 1);
     mbar_init_fence();
@@ -920,20 +933,22 @@ cudaError_t launch_spans(const Job& job, int vec_bytes, int grid, bool link, cud
     grid = grid > 0 ? (int)std::min<uint32_t>((uint32_t)grid, n) : (int)n;
     const bool retrieve = job.mode == MODE_RETRIEVE;
     const bool runs16 = dc.run_bytes % 16 == 0, narrow = has_narrow(job, vec_bytes);
-    if (runs16 && link) {
-        auto k = retrieve ? (narrow ? kvs_link_span_kernel<MODE_RETRIEVE, true> : kvs_link_span_kernel<MODE_RETRIEVE, false>)
-                          : (narrow ? kvs_link_span_kernel<MODE_STORE, true> : kvs_link_span_kernel<MODE_STORE, false>);
-        k<<<grid, kLdgThreads, 0, s>>>(dc, n);
-    } else if (runs16) {
-        auto k = retrieve ? (narrow ? kvs_span_kernel<MODE_RETRIEVE, true> : kvs_span_kernel<MODE_RETRIEVE, false>)
-                          : (narrow ? kvs_span_kernel<MODE_STORE, true> : kvs_span_kernel<MODE_STORE, false>);
-        k<<<grid, kSpanThreads, 0, s>>>(dc, n);
-    }
-    if (narrow) {
-        auto k = retrieve ? kvs_span_narrow_kernel<MODE_RETRIEVE> : kvs_span_narrow_kernel<MODE_STORE>;
-        k<<<grid, kSpanThreads, 0, s>>>(dc, n);
-    }
-    return cudaGetLastError();
+    return with_tables(job, [&](const auto& tab) {
+        constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+        if (runs16 && link) {
+            auto k = retrieve ? (narrow ? kvs_link_span_kernel<MODE_RETRIEVE, true, I> : kvs_link_span_kernel<MODE_RETRIEVE, false, I>)
+                              : (narrow ? kvs_link_span_kernel<MODE_STORE, true, I> : kvs_link_span_kernel<MODE_STORE, false, I>);
+            k<<<grid, kLdgThreads, 0, s>>>(dc, tab, n);
+        } else if (runs16) {
+            auto k = retrieve ? (narrow ? kvs_span_kernel<MODE_RETRIEVE, true, I> : kvs_span_kernel<MODE_RETRIEVE, false, I>)
+                              : (narrow ? kvs_span_kernel<MODE_STORE, true, I> : kvs_span_kernel<MODE_STORE, false, I>);
+            k<<<grid, kSpanThreads, 0, s>>>(dc, tab, n);
+        }
+        if (narrow) {
+            auto k = retrieve ? kvs_span_narrow_kernel<MODE_RETRIEVE, I> : kvs_span_narrow_kernel<MODE_STORE, I>;
+            k<<<grid, kSpanThreads, 0, s>>>(dc, tab, n);
+        }
+    });
 }
 
 cudaError_t launch_compare(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
@@ -955,7 +970,7 @@ cudaError_t launch_compare(const Job& job, int vec_bytes, int grid, cudaStream_t
 int link_ctas_per_sm() {
     static int n = 0;
     if (n == 0) {
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kvs_link_kernel<MODE_RETRIEVE>, kLdgThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kvs_link_kernel<MODE_RETRIEVE, false>, kLdgThreads, 0);
         if (n <= 0) n = 1;
     }
     return n;
@@ -1002,12 +1017,11 @@ cudaError_t launch_link(const Job& job, int vec_bytes, int grid, cudaStream_t s)
         return launch_spans(job, vec_bytes, clamp_grid(grid, 2, UINT64_MAX), true, s);
     grid = clamp_grid(grid, link_ctas_per_sm(), job.num_pieces);
     const Decoder dc = make_decoder(job);
-    const uint32_t n = (uint32_t)job.num_pieces;
-    if (job.mode == MODE_RETRIEVE)
-        kvs_link_kernel<MODE_RETRIEVE><<<grid, kLdgThreads, 0, s>>>(dc, n);
-    else
-        kvs_link_kernel<MODE_STORE><<<grid, kLdgThreads, 0, s>>>(dc, n);
-    return cudaGetLastError();
+    return with_tables(job, [&](const auto& tab) {
+        constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+        auto k = job.mode == MODE_RETRIEVE ? kvs_link_kernel<MODE_RETRIEVE, I> : kvs_link_kernel<MODE_STORE, I>;
+        k<<<grid, kLdgThreads, 0, s>>>(dc, tab, (uint32_t)job.num_pieces);
+    });
 }
 
 int ldg_ctas_per_sm() {
@@ -1031,12 +1045,11 @@ cudaError_t launch_ldg(const Job& job, int vec_bytes, int grid, cudaStream_t s) 
     if (job.mode == MODE_COMPARE) return launch_compare(job, vec_bytes, grid, s);
     if (vec_bytes == 16 && grid <= 0 && (uint64_t)job.block_size * job.row_bytes >= kPieceBytes / 2) {
         const Decoder dc = make_decoder(job);
-        const uint32_t n = (uint32_t)job.num_pieces;
-        if (job.mode == MODE_RETRIEVE)
-            kvs_ldg_piece_kernel<MODE_RETRIEVE><<<n, kPieceThreads, 0, s>>>(dc);
-        else
-            kvs_ldg_piece_kernel<MODE_STORE><<<n, kPieceThreads, 0, s>>>(dc);
-        return cudaGetLastError();
+        return with_tables(job, [&](const auto& tab) {
+            constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+            auto k = job.mode == MODE_RETRIEVE ? kvs_ldg_piece_kernel<MODE_RETRIEVE, I> : kvs_ldg_piece_kernel<MODE_STORE, I>;
+            k<<<(uint32_t)job.num_pieces, kPieceThreads, 0, s>>>(dc, tab);
+        });
     }
     return launch_spans(job, vec_bytes, grid > 0 ? clamp_grid(grid, kSpanCtasPerSm, job.num_pieces) : 0, false, s);
 }
@@ -1053,20 +1066,24 @@ cudaError_t launch_tma(const Job& job, int grid, cudaStream_t s) {
         // The carveout preference asks for the largest shared-memory split, so
         // that six 33 KiB CTAs (stage + reserved) fit on an SM.
         if (!g_tma_piece_cfg[dev]) {
-            for (auto fn : {kvs_tma_piece_kernel<MODE_RETRIEVE>, kvs_tma_piece_kernel<MODE_STORE>}) {
-                cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                                     (int)cudaSharedmemCarveoutMaxShared);
-                if (e != cudaSuccess) return e;
-            }
+            cudaError_t e = cudaSuccess;
+            auto prefer = [&](auto fn) {
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+            };
+            prefer(kvs_tma_piece_kernel<MODE_RETRIEVE, false>);
+            prefer(kvs_tma_piece_kernel<MODE_RETRIEVE, true>);
+            prefer(kvs_tma_piece_kernel<MODE_STORE, false>);
+            prefer(kvs_tma_piece_kernel<MODE_STORE, true>);
+            if (e != cudaSuccess) return e;
             g_tma_piece_cfg[dev] = true;
         }
         const Decoder dc = make_decoder(job);
-        const uint32_t n = (uint32_t)job.num_pieces;
-        if (job.mode == MODE_RETRIEVE)
-            kvs_tma_piece_kernel<MODE_RETRIEVE><<<n, 32, job.piece_bytes, s>>>(dc);
-        else
-            kvs_tma_piece_kernel<MODE_STORE><<<n, 32, job.piece_bytes, s>>>(dc);
-        return cudaGetLastError();
+        return with_tables(job, [&](const auto& tab) {
+            constexpr bool I = std::decay_t<decltype(tab)>::kInline;
+            auto k = job.mode == MODE_RETRIEVE ? kvs_tma_piece_kernel<MODE_RETRIEVE, I> : kvs_tma_piece_kernel<MODE_STORE, I>;
+            k<<<(uint32_t)job.num_pieces, 32, job.piece_bytes, s>>>(dc, tab);
+        });
     }
     const size_t smem = (size_t)kTmaStages * job.piece_bytes;
     if (g_tma_smem[dev] < smem) {             // the attribute is set per device

@@ -280,13 +280,23 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     int rc = scratch_address(&dscratch);
     if (rc) return rc;
     unsigned char* d = (unsigned char*)dscratch;
-    const size_t upload = validate && any_demoted ? need : off_bc;
-    NA_CUDA(cudaMemsetAsync(d, 0, sizeof(int32_t), s));             // error word starts at zero
-    NA_CUDA(cudaMemcpyAsync(d + off_pl, st + off_pl, upload - off_pl, cudaMemcpyHostToDevice, s));
+    // Small tables go in the launches' parameters (as in kvs_retrieve); the error word
+    // is read by validated calls only.
+    const HostTables tables{planes, entries, blocks, (uint32_t)P, (uint32_t)nent, (uint32_t)nrefs};
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    const cudaError_t capture = cudaStreamIsCapturing(s, &cs);
+    if (capture != cudaSuccess) cudaGetLastError();
+    const bool carried = !validate && tables_fit(tables) && capture == cudaSuccess && cs == cudaStreamCaptureStatusNone;
+    if (!carried) {
+        const size_t upload = validate && any_demoted ? need : off_bc;
+        NA_CUDA(cudaMemsetAsync(d, 0, sizeof(int32_t), s));             // error word starts at zero
+        NA_CUDA(cudaMemcpyAsync(d + off_pl, st + off_pl, upload - off_pl, cudaMemcpyHostToDevice, s));
+    }
 
     int vec = 16;
     while (vec > 1 && (addr_or & (uint64_t)(vec - 1))) vec >>= 1;
     Job j{};
+    j.tables = carried ? &tables : nullptr;
     j.entries = (const Entry*)(d + off_en);
     j.blocks = (const int32_t*)(d + off_bl);
     j.planes = (const uint64_t*)(d + off_pl);

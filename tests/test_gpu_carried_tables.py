@@ -1,0 +1,74 @@
+"""Calls whose tables travel in the launches' parameters, beside calls that upload them.
+
+Tables of up to 3584 bytes are carried; the sizes here lie on both sides of that, and
+calls of both kinds alternate without waiting, so that a table reused too early would
+show.  Exact equality with the CPU oracle.
+"""
+import pytest
+import torch
+
+import gpu_check as gc
+from paper_2609_35065_gb300 import buffers, kvs, synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _cuda():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    yield
+    torch.cuda.synchronize()
+
+
+def _table_bytes(w):
+    g = w.geom
+    entries = sum(len(w.chunk_counts(r)) for r in w.requests)
+    return 2 * g.layers * 8 + entries * 16 + entries * (g.chunk_tokens // g.block_size) * 4 + 8
+
+
+def _workload(requests, seed, residency, tokens=500):
+    return synth.custom(3, 2, 64, 16, 256, 400, [tokens] * requests, [tokens] * requests, seed=seed, residency=residency)
+
+
+@pytest.mark.parametrize("residency", ["host", "device", "mixed"])
+def test_tables_around_the_limit(residency):
+    """11, 21, 22 and 23 requests of two chunks (160 bytes a request): below, at and above."""
+    sizes = []
+    for n in (11, 21, 22, 23):
+        res = residency if residency != "mixed" else ["host", "device"] * (n // 2) + ["host"] * (n % 2)
+        w = synth.custom(3, 2, 64, 16, 256, n * 20, [300] * n, [300] * n, seed=n, residency=res)
+        sizes.append(_table_bytes(w))
+        buf = buffers.allocate(w)
+        kvs.kvs_retrieve(w.geom, buf.plane_ptrs, w.num_blocks, buf.requests, None)
+        torch.cuda.synchronize()
+        gc.check_retrieve(buf)
+    assert sizes[0] < 3584 < sizes[-1]
+
+
+@pytest.mark.parametrize("residency", ["host", "device"])
+def test_many_calls_in_flight(residency):
+    """Forty calls of different tables queued behind a sleeping kernel, every third uploaded."""
+    bufs = [buffers.allocate(_workload(24 if k % 3 == 0 else 1 + k % 4, k, residency, 40 + k)) for k in range(40)]
+    assert any(_table_bytes(b.workload) > 3584 for b in bufs) and any(_table_bytes(b.workload) < 3584 for b in bufs)
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(20_000_000)
+    for b in bufs:
+        kvs.kvs_retrieve(b.workload.geom, b.plane_ptrs, b.workload.num_blocks, b.requests, s)
+    s.synchronize()
+    for b in bufs:
+        gc.check_retrieve(b)
+
+
+@pytest.mark.parametrize("lps", [1, 2])
+def test_layer_groups_that_carry_and_that_upload(lps):
+    """20 layers: 20 launches upload, 10 with two layers each too; 3 layers carry."""
+    for L in (3, 20):
+        w = synth.custom(L, 2, 64, 16, 256, 60, [300], [300], seed=L, residency="device")
+        buf = buffers.allocate(w)
+        kvs.kvs_retrieve_layers(w.geom, buf.plane_ptrs, w.num_blocks, buf.requests, lps, None, None)
+        torch.cuda.synchronize()
+        gc.check_retrieve(buf)
