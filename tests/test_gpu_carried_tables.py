@@ -29,7 +29,7 @@ def _table_bytes(w):
 
 
 def _workload(requests, seed, residency, tokens=500):
-    return synth.custom(3, 2, 64, 16, 256, 400, [tokens] * requests, [tokens] * requests, seed=seed, residency=residency)
+    return synth.custom(3, 2, 64, 16, 256, 600, [tokens] * requests, [tokens] * requests, seed=seed, residency=residency)
 
 
 @pytest.mark.parametrize("residency", ["host", "device", "mixed"])
@@ -50,7 +50,7 @@ def test_tables_around_the_limit(residency):
 @pytest.mark.parametrize("residency", ["host", "device"])
 def test_many_calls_in_flight(residency):
     """Forty calls of different tables queued behind a sleeping kernel, every third uploaded."""
-    bufs = [buffers.allocate(_workload(24 if k % 3 == 0 else 1 + k % 4, k, residency, 40 + k)) for k in range(40)]
+    bufs = [buffers.allocate(_workload(24 if k % 3 == 0 else 1 + k % 4, k, residency, 280 + k)) for k in range(40)]
     assert any(_table_bytes(b.workload) > 3584 for b in bufs) and any(_table_bytes(b.workload) < 3584 for b in bufs)
     torch.cuda.synchronize()
     s = torch.cuda.Stream()
