@@ -1,15 +1,19 @@
-"""Build ``libkvs.so`` (the C-ABI library) in-tree with nvcc for sm_103a.
+"""Build ``libkvs.so`` (the C-ABI library) in-tree with nvcc for sm_103a, and the Python
+binding's marshalling extension beside it.
 
-``python -m paper_2609_35065_gb300.build`` or ``build_library()``.  The library
-lands in ``paper_2609_35065_gb300/_build/libkvs.so`` (git-ignored); it is
-rebuilt when a source or the public header is newer than it.
+``python -m paper_2609_35065_gb300.build`` or ``build_library()``.  Both land in
+``paper_2609_35065_gb300/_build/`` (git-ignored) and are rebuilt when a source or the
+public header is newer.  The extension needs Python's headers; without them the binding
+marshals with numpy and ctypes only.
 """
 from __future__ import annotations
 
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -24,6 +28,14 @@ DEPS = SOURCES + [os.path.join(CSRC, "kvs_internal.h"), os.path.join(CSRC, "kvs_
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 
+PYCALL_SOURCE = os.path.join(CSRC, "kvs_pycall.c")
+PYCALL = os.path.join(OUT_DIR, "kvs_pycall" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))
+
+
+def _has_python_headers() -> bool:
+    return os.path.exists(os.path.join(sysconfig.get_paths()["include"], "Python.h"))
+
+
 def nvcc() -> str:
     for cand in (shutil.which("nvcc"), "/usr/local/cuda/bin/nvcc"):
         if cand and os.path.exists(cand):
@@ -36,15 +48,55 @@ def command(out: str = LIB, extra: list[str] | None = None) -> list[str]:
             "-shared", "--threads", "4", "-I", INCLUDE, *SOURCES, "-o", out, *(extra or [])]
 
 
-def stale(out: str = LIB) -> bool:
+def pycall_command(out: str = PYCALL) -> list[str]:
+    cc = shutil.which("gcc") or shutil.which("cc")
+    if cc is None:
+        raise RuntimeError("a C compiler is required to build the binding's extension")
+    return [cc, "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-I", INCLUDE,
+            PYCALL_SOURCE, "-o", out]
+
+
+def _older(out: str, deps) -> bool:
     if not os.path.exists(out):
         return True
     t = os.path.getmtime(out)
-    return any(os.path.getmtime(d) > t for d in DEPS)
+    return any(os.path.getmtime(d) > t for d in deps)
+
+
+def stale(out: str = LIB) -> bool:
+    return _older(out, DEPS)
+
+
+def pycall_stale() -> bool:
+    return _has_python_headers() and _older(PYCALL, [PYCALL_SOURCE, os.path.join(INCLUDE, "kvs.h")])
+
+
+def load_pycall():
+    """The extension's ``call``, built first if its source is newer; None without Python's headers."""
+    if pycall_stale():
+        build_pycall()
+    if not os.path.exists(PYCALL):
+        return None
+    spec = importlib.util.spec_from_file_location("kvs_pycall", PYCALL)
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    return mod.call
+
+
+def build_pycall(verbose: bool = False) -> None:
+    os.makedirs(OUT_DIR, exist_ok=True)
+    tmp = PYCALL + f".{os.getpid()}.tmp"
+    cmd = pycall_command(tmp)
+    if verbose:
+        print(" ".join(cmd), file=sys.stderr)
+    subprocess.run(cmd, check=True)
+    os.replace(tmp, PYCALL)
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
+    if pycall_stale() or (force and _has_python_headers()):
+        build_pycall(verbose)
     if force or stale():
         tmp = LIB + f".{os.getpid()}.tmp"
         cmd = command(tmp)

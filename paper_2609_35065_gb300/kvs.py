@@ -1,8 +1,10 @@
-"""Python binding of the C ABI in ``include/kvs.h`` (ctypes; argument marshalling only).
+"""Python binding of the C ABI in ``include/kvs.h`` (argument marshalling only).
 
 Every function has the C name and forwards to ``libkvs.so``; every byte is moved
 by the library's CUDA kernels or copy-engine transfers.  There is no fallback:
-if the library cannot be loaded, :func:`lib` raises.
+if the library cannot be loaded, :func:`lib` raises.  The retrieval and store-back
+calls marshal ordinary arguments in a CPython extension (``csrc/kvs_pycall.c``) and
+anything else with numpy and ctypes, as all other functions do.
 
 Buffers are passed as integer addresses or as objects with ``data_ptr()``
 (torch tensors).  Streams are passed as integer ``cudaStream_t`` handles,
@@ -153,6 +155,8 @@ class kvs_tier_stats(ctypes.Structure):
 # ---- library loading ------------------------------------------------------
 _lock = threading.Lock()
 _lib = None
+_pycall = None              # the extension's call(), once the library is loaded
+_address: dict = {}         # addresses of the functions it may call
 
 
 def lib_path() -> str:
@@ -161,7 +165,9 @@ def lib_path() -> str:
 
 def lib():
     """Load ``libkvs.so`` (building it first if sources are newer).  Raises if impossible."""
-    global _lib
+    global _lib, _pycall
+    if _lib is not None:
+        return _lib
     with _lock:
         if _lib is None:
             path = lib_path()
@@ -233,6 +239,10 @@ def lib():
             L.kvs_stat_launches.restype = ctypes.c_int64
             L.kvs_selftest_wait_timeout.argtypes = [P, ctypes.c_int64]
             L.kvs_selftest_wait_timeout.restype = ctypes.c_int
+            for name in ("kvs_retrieve", "kvs_store", "kvs_retrieve_noalloc", "kvs_retrieve_fp8", "kvs_store_fp8",
+                         "kvs_retrieve_layers", "kvs_store_layers", "kvs_retrieve_fp8_layers", "kvs_store_fp8_layers"):
+                _address[name] = ctypes.cast(getattr(L, name), P).value
+            _pycall = _build.load_pycall()
             _lib = L
     return _lib
 
@@ -336,30 +346,50 @@ def _check(rc: int) -> int:
     return rc
 
 
-# ---- the C ABI, same names ------------------------------------------------
-def kvs_retrieve(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
-    """Enqueue retrieval of ``requests`` (list of :class:`RequestArg`) into the 2L
-    ``planes`` on ``stream``.  Raises :class:`KvsError` on a non-zero status."""
+def _whole_call(name, geom, planes, num_blocks, requests, stream, flags) -> int:
+    L = lib()
+    if _pycall is not None:
+        rc = _pycall(_address[name], geom if type(geom) is tuple else _geometry(geom), planes, num_blocks,
+                     requests, _stream(stream), flags)
+        if rc is not None:
+            return _check(rc)
     g = _geometry(geom)
     m = _Marshalled(planes, num_blocks, requests)
-    return _check(lib().kvs_retrieve(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                     _stream(stream), ctypes.c_uint32(flags)))
+    return _check(getattr(L, name)(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
+                                   _stream(stream), ctypes.c_uint32(flags)))
 
 
-def kvs_store(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
-    """Enqueue store-back of ``requests`` from the planes into their chunk buffers."""
+def _event_array(handles):
+    if handles is None:
+        return None, None
+    arr = (ctypes.c_void_p * max(1, len(handles)))(*handles)
+    return arr, ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p))
+
+
+def _layers_call(name, geom, planes, num_blocks, requests, layers_per_step, ready, events, stream, flags) -> int:
+    """``ready`` and ``events``: lists of cudaEvent_t handles, or None."""
+    L = lib()
+    store = "store" in name
+    if _pycall is not None:
+        rc = _pycall(_address[name], geom if type(geom) is tuple else _geometry(geom), planes, num_blocks,
+                     requests, _stream(stream), flags, 2 if store else 1, layers_per_step, ready, events)
+        if rc is not None:
+            return _check(rc)
     g = _geometry(geom)
     m = _Marshalled(planes, num_blocks, requests)
-    return _check(lib().kvs_store(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                  _stream(stream), ctypes.c_uint32(flags)))
+    keep_r, rev = _event_array(ready)
+    keep, ev = _event_array(events)
+    arrays = (rev, ev) if store else (ev,)
+    return _check(getattr(L, name)(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n, int(layers_per_step),
+                                   *arrays, _stream(stream), ctypes.c_uint32(flags)))
 
 
-def _events(events, stream):
+def _events(events):
     """cudaEvent_t handles of ``events``.  torch creates an event's handle at its first
     record, so a fresh ``torch.cuda.Event`` is first recorded once on the current
     stream; the library's record, made later in host order, is the one that waits see."""
     if events is None:
-        return None, None
+        return None
     handles = []
     for e in events:
         if e is None:
@@ -371,41 +401,44 @@ def _events(events, stream):
             handles.append(int(e.cuda_event))
         else:
             handles.append(int(e))
-    arr = (ctypes.c_void_p * max(1, len(handles)))(*handles)
-    return arr, ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p))
-
-
-def kvs_retrieve_layers(geom, planes, num_blocks, requests, layers_per_step, layer_events=None,
-                        stream=None, flags: int = 0) -> int:
-    """Layer-wise :func:`kvs_retrieve`: ``layer_events[k]`` (``torch.cuda.Event`` or raw
-    ``cudaEvent_t``) is recorded on ``stream`` after layer group k is enqueued."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    keep, ev = _events(layer_events, stream)
-    return _check(lib().kvs_retrieve_layers(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                            int(layers_per_step), ev, _stream(stream), ctypes.c_uint32(flags)))
+    return handles
 
 
 def _wait_events(events):
     """cudaEvent_t handles of events to wait on; an event never recorded (no handle yet)
     has nothing to wait for and is passed as NULL."""
     if events is None:
-        return None, None
-    handles = [0 if e is None else int(e.cuda_event) if hasattr(e, "cuda_event") else int(e) for e in events]
-    arr = (ctypes.c_void_p * max(1, len(handles)))(*handles)
-    return arr, ctypes.cast(arr, ctypes.POINTER(ctypes.c_void_p))
+        return None
+    return [0 if e is None else int(e.cuda_event) if hasattr(e, "cuda_event") else int(e) for e in events]
+
+
+# ---- the C ABI, same names ------------------------------------------------
+def kvs_retrieve(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
+    """Enqueue retrieval of ``requests`` (list of :class:`RequestArg`) into the 2L
+    ``planes`` on ``stream``.  Raises :class:`KvsError` on a non-zero status."""
+    return _whole_call("kvs_retrieve", geom, planes, num_blocks, requests, stream, flags)
+
+
+def kvs_store(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
+    """Enqueue store-back of ``requests`` from the planes into their chunk buffers."""
+    return _whole_call("kvs_store", geom, planes, num_blocks, requests, stream, flags)
+
+
+def kvs_retrieve_layers(geom, planes, num_blocks, requests, layers_per_step, layer_events=None,
+                        stream=None, flags: int = 0) -> int:
+    """Layer-wise :func:`kvs_retrieve`: ``layer_events[k]`` (``torch.cuda.Event`` or raw
+    ``cudaEvent_t``) is recorded on ``stream`` after layer group k is enqueued."""
+    return _layers_call("kvs_retrieve_layers", geom, planes, num_blocks, requests, layers_per_step, None,
+                        _events(layer_events), stream, flags)
 
 
 def kvs_store_layers(geom, planes, num_blocks, requests, layers_per_step, layer_events=None,
                      stream=None, flags: int = 0, ready_events=None) -> int:
     """Layer-wise :func:`kvs_store`: group k waits on ``ready_events[k]`` (recorded by the
     caller once those layers' KV is computed) and records ``layer_events[k]`` when copied."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    keep_r, rev = _wait_events(ready_events)
-    keep, ev = _events(layer_events, stream)
-    return _check(lib().kvs_store_layers(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                         int(layers_per_step), rev, ev, _stream(stream), ctypes.c_uint32(flags)))
+    ready = _wait_events(ready_events)
+    return _layers_call("kvs_store_layers", geom, planes, num_blocks, requests, layers_per_step, ready,
+                        _events(layer_events), stream, flags)
 
 
 def kvs_query_bw(stream=None, probe_bytes: int = 0) -> dict:
@@ -469,48 +502,33 @@ def kvs_retrieve_noalloc(geom, planes, num_blocks, requests, stream=None, flags:
     """Like :func:`kvs_retrieve`, for callers that cannot let the library allocate GPU
     memory: its scratch is a static device array of KVS_NOALLOC_SCRATCH_BYTES, so the
     call allocates nothing; calls that overlap on the GPU race on that array."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    return _check(lib().kvs_retrieve_noalloc(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                             _stream(stream), ctypes.c_uint32(flags)))
+    return _whole_call("kvs_retrieve_noalloc", geom, planes, num_blocks, requests, stream, flags)
 
 
 def kvs_retrieve_fp8(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
     """Dequantising retrieval from fp8 chunks (E4M3 codes with per-head scales) into
     BF16 planes; chunk buffers are [scales][codes], see kvs.h."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    return _check(lib().kvs_retrieve_fp8(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                         _stream(stream), ctypes.c_uint32(flags)))
+    return _whole_call("kvs_retrieve_fp8", geom, planes, num_blocks, requests, stream, flags)
 
 
 def kvs_store_fp8(geom, planes, num_blocks, requests, stream=None, flags: int = 0) -> int:
     """Quantising store-back from BF16 planes into fp8 chunks (scales and codes written)."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    return _check(lib().kvs_store_fp8(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                      _stream(stream), ctypes.c_uint32(flags)))
+    return _whole_call("kvs_store_fp8", geom, planes, num_blocks, requests, stream, flags)
 
 
 def kvs_retrieve_fp8_layers(geom, planes, num_blocks, requests, layers_per_step, layer_events=None,
                             stream=None, flags: int = 0) -> int:
     """Layer-wise :func:`kvs_retrieve_fp8`; ``layer_events[k]`` is recorded after group k."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    keep, ev = _events(layer_events, stream)
-    return _check(lib().kvs_retrieve_fp8_layers(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                                int(layers_per_step), ev, _stream(stream), ctypes.c_uint32(flags)))
+    return _layers_call("kvs_retrieve_fp8_layers", geom, planes, num_blocks, requests, layers_per_step, None,
+                        _events(layer_events), stream, flags)
 
 
 def kvs_store_fp8_layers(geom, planes, num_blocks, requests, layers_per_step, layer_events=None,
                          stream=None, flags: int = 0, ready_events=None) -> int:
     """Layer-wise :func:`kvs_store_fp8`: group k waits on ``ready_events[k]``."""
-    g = _geometry(geom)
-    m = _Marshalled(planes, num_blocks, requests)
-    keep_r, rev = _wait_events(ready_events)
-    keep, ev = _events(layer_events, stream)
-    return _check(lib().kvs_store_fp8_layers(ctypes.byref(g), ctypes.byref(m.cache), m.reqs, m.n,
-                                             int(layers_per_step), rev, ev, _stream(stream), ctypes.c_uint32(flags)))
+    ready = _wait_events(ready_events)
+    return _layers_call("kvs_store_fp8_layers", geom, planes, num_blocks, requests, layers_per_step, ready,
+                        _events(layer_events), stream, flags)
 
 
 # ---- fast tier ------------------------------------------------------------
