@@ -192,7 +192,8 @@ struct Plan {
     std::vector<int32_t>  blocks_cmp;    // KVS_F_VALIDATE: the demoted writers, compared
     std::vector<uint64_t> entry_bytes;   // bytes of each entry's chunk buffer
     uint32_t num_device = 0, num_host = 0;
-    uint32_t bpc = 0;
+    uint32_t bpc = 0;                    // blocks of the call's longest chunk
+    int32_t  max_tok = 0;                // its tokens
     uint64_t row_bytes = 0;
     uint64_t addr_or = 0;                // OR of all addresses and strides (alignment)
     uint64_t span_or = 0;                // the same with each chunk's n_tok * R for the row (Job::align)
@@ -229,7 +230,6 @@ int validate_call(const kvs_geometry* g, const kvs_paged_cache* cache,
     const int L = g->num_layers, B = g->block_size, C = g->chunk_tokens;
     const int P = 2 * L;
     pl.row_bytes = (uint64_t)g->num_kv_heads * g->head_dim * g->elem_bytes;
-    pl.bpc = (uint32_t)((C + B - 1) / B);
     pl.addr_or = pl.row_bytes;
     pl.planes.resize(P);
     for (int p = 0; p < P; ++p) {
@@ -260,6 +260,7 @@ int validate_call(const kvs_geometry* g, const kvs_paged_cache* cache,
             if (j + 1 < q.num_chunks && c.num_tokens != C)
                 return fail(KVS_ERR_INVALID_ARG, "request %d chunk %d: only the last chunk may be partial", r, j);
             sum += c.num_tokens;
+            pl.max_tok = std::max(pl.max_tok, c.num_tokens);
             if (c.residency == KVS_SRC_DEVICE) ++pl.num_device; else ++pl.num_host;
         }
         if (sum != q.num_tokens)
@@ -281,7 +282,10 @@ int validate_call(const kvs_geometry* g, const kvs_paged_cache* cache,
     }
 
     const uint32_t nent = pl.num_device + pl.num_host;
-    const uint64_t runs = (uint64_t)nent * P * pl.bpc;
+    // Pieces are laid out for the call's longest chunk, so that a call of short chunks (prompts
+    // below chunk_tokens) has no empty ones; the limit on a call's size is that of full chunks.
+    pl.bpc = (uint32_t)((pl.max_tok + B - 1) / B);
+    const uint64_t runs = (uint64_t)nent * P * (uint64_t)((C + B - 1) / B);
     const uint64_t ppr = ((uint64_t)B * pl.row_bytes + kPieceBytes - 1) / kPieceBytes;
     if (runs * ppr >= (1ull << 31))
         return fail(KVS_ERR_INVALID_ARG, "call too large: split it (more than 2^31 pieces)");
@@ -1017,7 +1021,7 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
         f.rows_whole = (kFp8PieceCodes / 16) % (hd / 16) == 0;
         const Entry& last = pl.entries[first + count - 1];
         f.tokens = (uint64_t)last.first_tok + (uint32_t)last.n_tok;
-        f.ragged = f.tokens != (uint64_t)count * (uint32_t)g->chunk_tokens;
+        f.ragged = f.tokens != (uint64_t)count * (uint32_t)pl.max_tok;
         return f;
     };
     // store-back segments: one per (chunk, plane, head)
@@ -1025,7 +1029,7 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
         return (uint64_t)f.job.num_entries * f.job.num_planes * f.heads;
     };
     auto run = [&](const Fp8Job& f, int grid, bool device_chunks) -> int {
-        cudaError_t e = !retrieve ? launch_fp8_store(f, grid, s, (uint32_t)g->chunk_tokens, device_chunks)
+        cudaError_t e = !retrieve ? launch_fp8_store(f, grid, s, (uint32_t)pl.max_tok, device_chunks)
                       : (few && !device_chunks) ? launch_fp8_retrieve_staged(f, grid, s)
                                                 : launch_fp8_retrieve(f, grid, s);
         if (e != cudaSuccess) return fail(KVS_ERR_CUDA, "fp8 kernel launch failed: %s", cudaGetErrorString(e));

@@ -132,7 +132,8 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
 
     const int L = g->num_layers, B = g->block_size, C = g->chunk_tokens, P = 2 * L;
     const uint64_t R = (uint64_t)g->num_kv_heads * g->head_dim * e_b;
-    const uint32_t bpc = (uint32_t)((C + B - 1) / B);
+    uint32_t bpc = (uint32_t)((C + B - 1) / B);
+    int32_t max_tok = 0;
     uint64_t addr_or = R, span_or = 0;
     for (int p = 0; p < P; ++p) {
         if (!cache->kv_planes[p]) return na_fail(KVS_ERR_INVALID_ARG, "plane %d is NULL", p);
@@ -161,6 +162,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
             if (j + 1 < q.num_chunks && c.num_tokens != C)
                 return na_fail(KVS_ERR_INVALID_ARG, "request %d chunk %d: only the last chunk may be partial", r, j);
             sum += c.num_tokens;
+            max_tok = std::max(max_tok, c.num_tokens);
             if (c.residency == KVS_SRC_DEVICE) ++ndev;
         }
         if (sum != q.num_tokens)
@@ -183,14 +185,14 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     }
     if (nent == 0) return KVS_OK;
 
-    // Scratch needed by this call: refuse anything beyond the static array.
+    // Scratch needed by this call, with every chunk counted as a full one: refuse anything beyond
+    // the static array.  The tables themselves are laid out for the call's longest chunk.
     const bool validate = flags & KVS_F_VALIDATE;
-    const uint64_t nrefs = nent * bpc;
     const size_t off_pl = 256;
     const size_t off_en = off_pl + up256((size_t)P * 8);
     const size_t off_bl = off_en + up256((size_t)nent * sizeof(Entry));
-    const size_t off_bc = off_bl + up256((size_t)nrefs * 4);
-    const size_t need = off_bc + (validate ? up256((size_t)nrefs * 4) : 0);
+    uint64_t nrefs = nent * bpc;
+    size_t need = off_bl + up256((size_t)nrefs * 4) * (validate ? 2 : 1);
     if (need > KVS_NOALLOC_SCRATCH_BYTES || nrefs > kMaxBlockRefs)
         return na_fail(KVS_ERR_UNSUPPORTED,
                        "this call needs %zu bytes of descriptor scratch; kvs_retrieve_noalloc holds at most %u "
@@ -199,6 +201,10 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     const uint64_t ppr = ((uint64_t)B * R + kPieceBytes - 1) / kPieceBytes;
     if (nrefs * P * ppr >= (1ull << 31))
         return na_fail(KVS_ERR_INVALID_ARG, "call too large: split it (more than 2^31 pieces)");
+    bpc = (uint32_t)((max_tok + B - 1) / B);
+    nrefs = nent * bpc;
+    const size_t off_bc = off_bl + up256((size_t)nrefs * 4);
+    need = off_bc + (validate ? up256((size_t)nrefs * 4) : 0);
 
     // Pack the tables: device-resident entries first, then host-resident ones,
     // so that each class is one contiguous range of entries (one launch each).

@@ -22,6 +22,7 @@ SHAPES = {
     "head_80": (2, 3, 80, 16, 256, (257, 40)),
     "head_176_rows_cross_pieces": (2, 5, 176, 3, 48, (200, 47)),
     "one_vector": (1, 1, 16, 1, 1, (1,)),
+    "all_chunks_short": (3, 2, 64, 16, 256, (42, 17, 33)),
 }
 
 

@@ -23,6 +23,7 @@ SHAPES = {
     "cluster_of_2": (2, 3, 256, 16, 256, (600, 255, 1)),
     "cluster_of_4": (2, 2, 512, 32, 256, (300, 512)),
     "cluster_of_2_odd_rows": (2, 1, 208, 1, 260, (520, 7)),
+    "all_chunks_short": (2, 8, 128, 16, 256, (42, 17, 33)),
     "above_every_unit": (1, 1, 1024, 16, 256, (300,)),       # falls to the two-pass kernel
 }
 

@@ -25,6 +25,8 @@ GEOMETRIES = {
     "long_runs": (1, 5, 300, 2, 16, 64, (200, 64)),                         # 48000-byte runs, two a piece
     "long_runs_odd_chunk": (1, 7, 333, 2, 16, 64, (197,)),                  # 74592-byte runs
     "one_vector": (1, 1, 8, 2, 1, 1, (1,)),
+    "all_chunks_short": (3, 2, 64, 2, 16, 256, (42, 17, 33)),
+    "all_chunks_short_32KiB_runs": (2, 8, 128, 2, 16, 256, (40, 1, 48)),
 }
 
 
