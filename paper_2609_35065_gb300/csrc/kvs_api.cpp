@@ -464,9 +464,9 @@ struct Uploaded {
     const HostTables* host = nullptr;
 };
 
-HostTables host_tables(const Plan& pl) {
+HostTables host_tables(const Plan& pl, bool forked) {
     return {pl.planes.data(), pl.entries.data(), pl.blocks.data(),
-            (uint32_t)pl.planes.size(), (uint32_t)pl.entries.size(), (uint32_t)pl.blocks.size()};
+            (uint32_t)pl.planes.size(), (uint32_t)pl.entries.size(), (uint32_t)pl.blocks.size(), forked};
 }
 
 // Whether a call's launches carry its tables.  An upload costs the call 3 to 4 us of
@@ -808,7 +808,7 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     const Mode mode = retrieve ? MODE_RETRIEVE : MODE_STORE;
     const int host_grid = grid ? grid : f_few ? st.few_sm_ctas : (retrieve ? st.hostlink_ctas : st.store_ctas);
 
-    const HostTables tables = host_tables(pl);
+    const HostTables tables = host_tables(pl, pl.num_device && pl.num_host);
     Uploaded u;
     const bool plain_host = !pl.num_host || (host_variant == KVS_VARIANT_HOSTLINK && !f_few &&
                                              !(flags & (KVS_F_PREFETCH_L2 | KVS_F_LAYER_SIGNAL)));
@@ -987,7 +987,7 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
     const int L = g->num_layers;
     const int lps = layers_per_step > 0 ? std::min(layers_per_step, L) : L;
     const int groups = (L + lps - 1) / lps;
-    const HostTables tables = host_tables(pl);
+    const HostTables tables = host_tables(pl, false);
     Uploaded u;
     if (!few && !(flags & KVS_F_VALIDATE) && carry_tables(tables, groups * ((pl.num_host > 0) + (pl.num_device > 0)), s)) {
         u.host = &tables;

@@ -290,6 +290,7 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint
 template <bool INL>
 __global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
 kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
+    if (INL) grid_wait();
     RtRegs<kRtLinkVec> ra, rb;
     Fp8Span pa, pb;
     uint32_t q = blockIdx.x;
@@ -311,6 +312,10 @@ kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_consta
 template <bool INL>
 __global__ void __launch_bounds__(kRtHbm, kRtHbmCtas)
 kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
+    if (INL) {
+        grid_wait();
+        grid_trigger();
+    }
     Fp8Span sp;
     if (!fp8_span(dc, tab, blockIdx.x, sp)) return;              // uniform across the CTA
     RtRegs<kRtHbmVec> r;
@@ -607,6 +612,7 @@ __device__ __forceinline__ void store_head_segment(const Fp8Job& f, const TAB& t
 template <bool INL>
 __global__ void __launch_bounds__(kStThreads)
 kvs_fp8_store_head_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t num_segments) {
+    if (INL) grid_wait();
     __shared__ uint32_t warp_max[kStThreads / 32];
     __shared__ float sm_inv;
     const Job& j = f.job;
@@ -750,6 +756,7 @@ __device__ __forceinline__ void cluster_sync() {
 template <int VEC, bool CLUSTER, bool INL>
 __global__ void __launch_bounds__(kUqThreads, uq_ctas(CLUSTER))
 kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t g, uint32_t G, uint32_t extra, uint32_t cl) {
+    if (INL) grid_wait();
     extern __shared__ __align__(128) uint8_t uq_smem[];
     uint32_t* rows = reinterpret_cast<uint32_t*>(uq_smem + uq_stage_bytes(VEC));   // plane row of each of the CTA's tokens
     // Maxima of unit n's heads in third n % 3, cleared before barrier n - 1: the readers of unit
@@ -881,6 +888,7 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, const __grid_constan
             src = source();
         } else {
             mine = 0;
+            if (INL) grid_trigger();
         }
         const uint64_t inv2 = ((uint64_t)__float_as_uint(inv) << 32) | __float_as_uint(inv);
 #pragma unroll
@@ -901,6 +909,7 @@ constexpr int kStUnroll = 4;                         // vectors per thread in fl
 template <bool INL>
 __global__ void __launch_bounds__(kStThreads)
 kvs_fp8_store_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ Tables<INL> tab, uint32_t num_segments) {
+    if (INL) grid_wait();
     __shared__ uint32_t amax[kFp8MaxHeads];
     __shared__ float scale[kFp8MaxHeads];                    // holds 448 / amax per head
     const Job& j = f.job;
@@ -1045,8 +1054,8 @@ cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s) {
     const uint32_t ctas = per_piece ? dc.num_pieces : std::min<uint32_t>((uint32_t)grid, dc.num_pieces);
     return with_tables(fj.job, [&](const auto& tab) {
         constexpr bool I = std::decay_t<decltype(tab)>::kInline;
-        if (per_piece) kvs_fp8_retrieve_piece_kernel<I><<<ctas, kRtHbm, 0, s>>>(dc, tab);
-        else kvs_fp8_retrieve_kernel<I><<<ctas, kRtLink, 0, s>>>(dc, tab);
+        if (per_piece) launch_on(s, tab, kvs_fp8_retrieve_piece_kernel<I>, ctas, kRtHbm, 0, dc, tab);
+        else launch_on(s, tab, kvs_fp8_retrieve_kernel<I>, ctas, kRtLink, 0, dc, tab);
     });
 }
 
@@ -1109,7 +1118,7 @@ cudaError_t launch_unit(const Fp8Job& fj, const Tables<INL>& tab, int grid, cuda
     cfg.blockDim = dim3(kUqThreads);
     cfg.dynamicSmemBytes = uq_stage_bytes(VEC) + (chunk_tokens + cl - 1) / cl * 4;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     if (CLUSTER) {                                          // as many clusters as the GPCs hold at once
         at[0].id = cudaLaunchAttributeClusterDimension;
         at[0].val.clusterDim.x = cl;
@@ -1132,6 +1141,12 @@ cudaError_t launch_unit(const Fp8Job& fj, const Tables<INL>& tab, int grid, cuda
     if ((uint64_t)ctas > units) ctas = (int)units;
     const uint32_t G = uq_team(fj.heads / g, (uint32_t)ctas);
     cfg.gridDim = dim3((uint32_t)ctas / G * G * cl);
+    if (tab.programmatic()) {                               // see launch_on
+        at[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[cfg.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = at;
+        ++cfg.numAttrs;
+    }
     const uint32_t extra = kUqUnitBytes / (g * fj.head_dim * 2);
     return cudaLaunchKernelEx(&cfg, k, fj, tab, g, G, extra, cl);
 }
@@ -1164,7 +1179,7 @@ cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_
         if (grid <= 0 || (uint64_t)grid > segs) grid = (int)std::min<uint64_t>(segs, 1u << 30);
         return with_tables(fj.job, [&](const auto& tab) {
             constexpr bool I = std::decay_t<decltype(tab)>::kInline;
-            kvs_fp8_store_head_kernel<I><<<grid, kStThreads, 0, s>>>(fj, tab, (uint32_t)segs);
+            launch_on(s, tab, kvs_fp8_store_head_kernel<I>, grid, kStThreads, 0, fj, tab, (uint32_t)segs);
         });
     }
     const uint64_t segs = (uint64_t)fj.job.num_entries * fj.job.num_planes;
@@ -1172,7 +1187,7 @@ cudaError_t launch_fp8_store(const Fp8Job& fj, int grid, cudaStream_t s, uint32_
     if (grid <= 0 || (uint64_t)grid > segs) grid = (int)segs;
     return with_tables(fj.job, [&](const auto& tab) {
         constexpr bool I = std::decay_t<decltype(tab)>::kInline;
-        kvs_fp8_store_kernel<I><<<grid, kStThreads, 0, s>>>(fj, tab, (uint32_t)segs);
+        launch_on(s, tab, kvs_fp8_store_kernel<I>, grid, kStThreads, 0, fj, tab, (uint32_t)segs);
     });
 }
 

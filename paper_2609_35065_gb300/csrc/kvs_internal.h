@@ -29,6 +29,7 @@ struct HostTables {
     const Entry*    entries;         // of all classes
     const int32_t*  blocks;
     uint32_t num_planes, num_entries, num_blocks;
+    uint32_t forked;                 // the call's launches run on two streams, between events
 };
 
 // What a launch can carry: with its other parameters within 4 KiB.

@@ -356,8 +356,10 @@ constexpr int kSpanUnroll = kPieceBytes / 16 / kSpanThreads;
 template <int MODE, bool TAIL, bool INL>
 __global__ void __launch_bounds__(kSpanThreads, TAIL ? 3 : kSpanCtasPerSm)
 kvs_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
+    if (INL) grid_wait();
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
+        if (INL && q + gridDim.x >= num_pieces) grid_trigger();
         if (!span_piece(dc, tab, q, sp)) continue;            // uniform across the CTA
         if (TAIL && !span_wide(dc, sp)) continue;
         uint4 r[kSpanUnroll];
@@ -373,8 +375,10 @@ kvs_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ 
 template <int MODE, bool INL>
 __global__ void __launch_bounds__(kSpanThreads, 3)
 kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
+    if (INL) grid_wait();
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
+        if (INL && q + gridDim.x >= num_pieces) grid_trigger();
         if (!span_piece(dc, tab, q, sp) || span_wide(dc, sp)) continue;   // uniform across the CTA
         const uint32_t a = (uint32_t)sp.chunk | (uint32_t)sp.plane | sp.off | (uint32_t)dc.run_bytes | sp.len;
         if ((a & 7) == 0) span_narrow<MODE, 8, 4>(dc, tab, sp);
@@ -394,6 +398,10 @@ constexpr int kPieceUnroll = kPieceBytes / 16 / kPieceThreads;
 template <int MODE, bool INL>
 __global__ void __launch_bounds__(kPieceThreads, 4)
 kvs_ldg_piece_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab) {
+    if (INL) {
+        grid_wait();
+        grid_trigger();
+    }
     static_assert(kPieceUnroll * kPieceThreads * 16 == kPieceBytes, "one piece per CTA");
     Piece pc;
     if (!decode_piece(dc, tab, blockIdx.x, pc)) return;  // uniform across the CTA
@@ -457,6 +465,7 @@ __device__ __forceinline__ void store_piece16(uint64_t dst, uint32_t len, const 
 template <int MODE, bool INL>
 __global__ void __launch_bounds__(kLdgThreads)
 kvs_link_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
+    if (INL) grid_wait();
     static_assert(kPieceBytes == kLdgUnroll * kLdgThreads * 16, "one piece per register set");
     constexpr bool to_plane = (MODE == MODE_RETRIEVE);
     uint4 ra[kLdgUnroll], rb[kLdgUnroll];
@@ -482,6 +491,7 @@ kvs_link_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tabl
 template <int MODE, bool TAIL, bool INL>
 __global__ void __launch_bounds__(kLdgThreads, 2)
 kvs_link_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
+    if (INL) grid_wait();
     uint4 ra[kLdgUnroll], rb[kLdgUnroll];
     int32_t ba[kLdgUnroll], bb[kLdgUnroll];
     SpanPiece pa, pb;
@@ -824,6 +834,10 @@ __global__ void __launch_bounds__(32, 1) kvs_tma_kernel(const Decoder dc, uint32
 template <int MODE, bool INL>
 __global__ void __launch_bounds__(32)
 kvs_tma_piece_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tables<INL> tab) {
+    if (INL) {
+        grid_wait();
+        grid_trigger();
+    }
     extern __shared__ __align__(128) uint8_t stage[];
     __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x != 0) return;
@@ -938,15 +952,15 @@ cudaError_t launch_spans(const Job& job, int vec_bytes, int grid, bool link, cud
         if (runs16 && link) {
             auto k = retrieve ? (narrow ? kvs_link_span_kernel<MODE_RETRIEVE, true, I> : kvs_link_span_kernel<MODE_RETRIEVE, false, I>)
                               : (narrow ? kvs_link_span_kernel<MODE_STORE, true, I> : kvs_link_span_kernel<MODE_STORE, false, I>);
-            k<<<grid, kLdgThreads, 0, s>>>(dc, tab, n);
+            launch_on(s, tab, k, grid, kLdgThreads, 0, dc, tab, n);
         } else if (runs16) {
             auto k = retrieve ? (narrow ? kvs_span_kernel<MODE_RETRIEVE, true, I> : kvs_span_kernel<MODE_RETRIEVE, false, I>)
                               : (narrow ? kvs_span_kernel<MODE_STORE, true, I> : kvs_span_kernel<MODE_STORE, false, I>);
-            k<<<grid, kSpanThreads, 0, s>>>(dc, tab, n);
+            launch_on(s, tab, k, grid, kSpanThreads, 0, dc, tab, n);
         }
         if (narrow) {
             auto k = retrieve ? kvs_span_narrow_kernel<MODE_RETRIEVE, I> : kvs_span_narrow_kernel<MODE_STORE, I>;
-            k<<<grid, kSpanThreads, 0, s>>>(dc, tab, n);
+            launch_on(s, tab, k, grid, kSpanThreads, 0, dc, tab, n);
         }
     });
 }
@@ -1020,7 +1034,7 @@ cudaError_t launch_link(const Job& job, int vec_bytes, int grid, cudaStream_t s)
     return with_tables(job, [&](const auto& tab) {
         constexpr bool I = std::decay_t<decltype(tab)>::kInline;
         auto k = job.mode == MODE_RETRIEVE ? kvs_link_kernel<MODE_RETRIEVE, I> : kvs_link_kernel<MODE_STORE, I>;
-        k<<<grid, kLdgThreads, 0, s>>>(dc, tab, (uint32_t)job.num_pieces);
+        launch_on(s, tab, k, grid, kLdgThreads, 0, dc, tab, (uint32_t)job.num_pieces);
     });
 }
 
@@ -1048,7 +1062,7 @@ cudaError_t launch_ldg(const Job& job, int vec_bytes, int grid, cudaStream_t s) 
         return with_tables(job, [&](const auto& tab) {
             constexpr bool I = std::decay_t<decltype(tab)>::kInline;
             auto k = job.mode == MODE_RETRIEVE ? kvs_ldg_piece_kernel<MODE_RETRIEVE, I> : kvs_ldg_piece_kernel<MODE_STORE, I>;
-            k<<<(uint32_t)job.num_pieces, kPieceThreads, 0, s>>>(dc, tab);
+            launch_on(s, tab, k, (uint32_t)job.num_pieces, kPieceThreads, 0, dc, tab);
         });
     }
     return launch_spans(job, vec_bytes, grid > 0 ? clamp_grid(grid, kSpanCtasPerSm, job.num_pieces) : 0, false, s);
@@ -1082,7 +1096,7 @@ cudaError_t launch_tma(const Job& job, int grid, cudaStream_t s) {
         return with_tables(job, [&](const auto& tab) {
             constexpr bool I = std::decay_t<decltype(tab)>::kInline;
             auto k = job.mode == MODE_RETRIEVE ? kvs_tma_piece_kernel<MODE_RETRIEVE, I> : kvs_tma_piece_kernel<MODE_STORE, I>;
-            k<<<(uint32_t)job.num_pieces, 32, job.piece_bytes, s>>>(dc, tab);
+            launch_on(s, tab, k, (uint32_t)job.num_pieces, 32, job.piece_bytes, dc, tab);
         });
     }
     const size_t smem = (size_t)kTmaStages * job.piece_bytes;

@@ -288,7 +288,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     unsigned char* d = (unsigned char*)dscratch;
     // Small tables go in the launches' parameters (as in kvs_retrieve); the error word
     // is read by validated calls only.
-    const HostTables tables{planes, entries, blocks, (uint32_t)P, (uint32_t)nent, (uint32_t)nrefs};
+    const HostTables tables{planes, entries, blocks, (uint32_t)P, (uint32_t)nent, (uint32_t)nrefs, 0};
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const cudaError_t capture = cudaStreamIsCapturing(s, &cs);
     if (capture != cudaSuccess) cudaGetLastError();
