@@ -487,7 +487,7 @@ kvs_link_kernel(const __grid_constant__ Decoder dc, const __grid_constant__ Tabl
 // The same over wide span pieces, for short runs and odd rows (TAIL as above).  A
 // run alone gives a 256-thread CTA run_bytes / 4096 vectors a thread, and the link
 // wants megabytes in flight: with 2 KiB runs, retrieval 340 -> 239 us and
-// store-back 279 -> 269 us at 49 MB (the link's own time: 233 and 254).
+// store-back 279 -> 259 us at 49 MB (the link's own time: 233 and 254).
 template <int MODE, bool TAIL, bool INL>
 __global__ void __launch_bounds__(kLdgThreads, 2)
 kvs_link_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
@@ -1025,9 +1025,9 @@ cudaError_t launch_link_staged(const Job& job, int grid, cudaStream_t s) {
 
 cudaError_t launch_link(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
     if (job.num_pieces == 0) return cudaSuccess;
-    // Short runs as span pieces.  98 MB retrieved in 4 KiB runs: 472 us against 482 by runs, in
-    // 8 KiB runs 474 either way; stored in 4 KiB runs: 534 against 523.
-    if (vec_bytes != 16 || (uint64_t)job.block_size * job.row_bytes < (job.mode == MODE_RETRIEVE ? 8192 : 4096))
+    // Short runs as span pieces.  98 MB in 4 KiB runs: 471 us retrieved and 513 stored, against 480
+    // and 524 by runs; in 8 KiB runs 471 and 513 either way.
+    if (vec_bytes != 16 || (uint64_t)job.block_size * job.row_bytes < 8192)
         return launch_spans(job, vec_bytes, clamp_grid(grid, 2, UINT64_MAX), true, s);
     grid = clamp_grid(grid, link_ctas_per_sm(), job.num_pieces);
     const Decoder dc = make_decoder(job);
