@@ -1125,11 +1125,16 @@ cudaError_t launch_unit(const Fp8Job& fj, const Tables<INL>& tab, int grid, cuda
         at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
         cfg.attrs = at;
         cfg.numAttrs = 1;
-        cfg.gridDim = dim3((uint32_t)full * cl);
-        int most = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&most, k, &cfg);
-        if (e != cudaSuccess) return e;
-        full = std::max(1, std::min(full, most));
+        static struct { uint32_t cl, smem; int most; } seen[kMaxDev];   // the last answer
+        auto& known = seen[dev];
+        if (known.cl != cl || known.smem != cfg.dynamicSmemBytes) {
+            cfg.gridDim = dim3((uint32_t)full * cl);
+            const cudaError_t e = cudaOccupancyMaxActiveClusters(&known.most, k, &cfg);
+            if (e != cudaSuccess) return e;
+            known.cl = cl;
+            known.smem = (uint32_t)cfg.dynamicSmemBytes;
+        }
+        full = std::max(1, std::min(full, known.most));
     }
     int ctas = grid > 0 ? std::max(1, std::min(grid / (int)cl, full)) : full;
     uint64_t units = 0;
