@@ -1045,16 +1045,15 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             const Fp8Job f = fjob(pl.num_device, pl.num_host, p0, np);
             if (f.job.num_pieces >= (1ull << 31) || fp8_segments(f) >= (1ull << 31))
                 return fail(KVS_ERR_INVALID_ARG, "call too large: split it");
-            // Retrieval: a CTA keeps up to 32 KiB of codes in flight, half a link-kernel
-            // CTA's bytes, so it takes twice the link kernel's grid.  Store-back: one CTA
-            // per (chunk, plane, head) over the whole GPU for a whole call (193 GB/s, the
-            // D2H link); layer by layer it runs beside the compute that produces the KV,
-            // where a whole-GPU launch per group displaces that compute, so it takes the
-            // host-link store cap (exposed store time per 8B prefill: 7.7 ms uncapped,
-            // 2.1 ms at 32 CTAs).
+            // Retrieval: an eighth more CTAs than the link kernel (see kvs_fp8_retrieve_kernel).
+            // Store-back: one CTA per (chunk, plane, head) over the whole GPU for a whole call
+            // (193 GB/s, the D2H link); layer by layer it runs beside the compute that produces
+            // the KV, where a whole-GPU launch per group displaces that compute, so it takes the
+            // host-link store cap (exposed store time per 8B prefill: 7.7 ms uncapped, 2.1 ms at
+            // 32 CTAs).
             // KVS_F_FEW_SMS: the staged kernel on the BF16 staged kernel's cap (each of its
             // CTAs holds 112 KiB of codes, about what a BF16 staged CTA holds).
-            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? 2 * st.hostlink_ctas
+            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? st.hostlink_ctas + st.hostlink_ctas / 8
                            : layers_per_step > 0 ? st.store_ctas : 0;
             rc = run(f, grid, false);
             if (rc) return rc;

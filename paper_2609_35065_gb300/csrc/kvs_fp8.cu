@@ -24,7 +24,7 @@
 // both signs and compares with the oracle).
 //
 // Retrieval is bound by the host link (or HBM for device chunks): a persistent
-// grid of 256-thread CTAs walks span pieces of 16 KiB of codes; each thread keeps two
+// grid of 512-thread CTAs walks span pieces of 16 KiB of codes; each thread keeps two
 // pieces' worth of 16-byte code vectors in registers, so the next piece's loads
 // are in flight while the current one is converted and stored.  HBM chunks run one
 // CTA per piece instead, and KVS_F_FEW_SMS runs a kernel that also stages pieces in
@@ -53,7 +53,7 @@ namespace {
 
 // Threads, 16-code vectors per thread per piece, and CTAs per SM of the retrieval
 // kernels: host chunks (two pieces in registers each), HBM chunks.
-constexpr int kRtLink = 256, kRtLinkVec = 4, kRtLinkCtas = 4;
+constexpr int kRtLink = 512, kRtLinkVec = 2, kRtLinkCtas = 2;
 constexpr int kRtHbm = 256, kRtHbmVec = 4, kRtHbmCtas = 6;
 static_assert(kRtLink * kRtLinkVec * 16 == kFp8PieceCodes && kRtHbm * kRtHbmVec * 16 == kFp8PieceCodes,
               "a piece is one vector set per CTA");
@@ -233,7 +233,7 @@ __device__ __forceinline__ void st_bf16x16(uint64_t a, const uint4& lo, const ui
 }
 
 // This thread's vectors of a piece in flight: codes, the scales of their heads, blocks
-// (-1: no such vector; one out of range, which the planner has excluded, is reported).
+// (after rt_check, -1 where there is nothing to move).
 template <int U>
 struct RtRegs {
     uint4   c[U];
@@ -244,7 +244,6 @@ struct RtRegs {
 template <int T, int U, class TAB>
 __device__ __forceinline__ void rt_load(const Fp8Spans& dc, const TAB& tab, const Fp8Span& sp, RtRegs<U>& r) {
     const uint32_t nv = sp.len / 16;
-    bool bad = false;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint32_t v = threadIdx.x + u * T;
@@ -252,11 +251,21 @@ __device__ __forceinline__ void rt_load(const Fp8Spans& dc, const TAB& tab, cons
         r.s[u] = __ldg(reinterpret_cast<const float*>(sp.scales) + fp8_vec_head(dc, sp, min(v, nv - 1)));
         r.blk[u] = tab.block(sp.run0 + fp8_run(dc, sp, min(v, nv - 1) * 16));
     }
+}
+
+// Waits for the blocks; one out of range, which the planner has excluded, is reported
+// and skipped.  A host-link CTA checks a piece only before it stores it, with the next
+// one's loads on the way (24 CTAs: 138 GB/s when it checked at once, 168 so); a CTA of
+// one piece checks at once, while its codes are on the way (8 x 2048 tokens from HBM: 464
+// us, 474 the other way).
+template <int T, int U>
+__device__ __forceinline__ void rt_check(const Fp8Spans& dc, const Fp8Span& sp, RtRegs<U>& r) {
+    bool bad = false;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const bool in = (uint32_t)r.blk[u] < (uint32_t)dc.f.job.num_blocks;
         bad |= !in && r.blk[u] >= 0;
-        if (!in || threadIdx.x + u * T >= nv) r.blk[u] = -1;
+        if (!in || threadIdx.x + u * T >= sp.len / 16) r.blk[u] = -1;
     }
     if (bad) atomicCAS(dc.f.job.err, 0, KVS_ERR_BOUNDS);
 }
@@ -282,11 +291,12 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint
     return false;
 }
 
-// Host chunks: the next piece's loads are in flight while a piece is converted.  64
-// registers, so that four CTAs, 128 KiB of codes, still share an SM beside a kernel
-// that leaves them few SMs.  8192 tokens of the 8B shape: 2561 us with 128 threads x
-// 8 vectors and scales through shared memory, 2570 without it, 2555 here (the link:
-// 2541); 512 x 2 gains another 0.1% but fits two CTAs per SM.
+// Host chunks: the next piece's loads are in flight while a piece is converted.  512
+// threads, so that a piece's conversion keeps the next one's loads waiting as little as
+// possible: 24 CTAs hold 207 GB/s alone, where 256 threads x 4 vectors hold 168 and 128
+// x 8 133 to 176.  8192 tokens of the 8B shape on the default grid: 2561 -> 2553 us (the
+// link: 2541).  Beside a GEMM loop 50 to 56 CTAs, two an SM, keep what 100 CTAs of 128
+// threads kept, four an SM: 200 against 201 GB/s with the GEMM at 88% either way.
 template <bool INL>
 __global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
 kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
@@ -299,10 +309,12 @@ kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_consta
     while (ha) {
         const bool hb = rt_next(dc, tab, q, pb);
         if (hb) rt_load<kRtLink>(dc, tab, pb, rb);
+        rt_check<kRtLink>(dc, pa, ra);
         rt_store<kRtLink>(dc, pa, ra);
         if (!hb) break;
         ha = rt_next(dc, tab, q, pa);
         if (ha) rt_load<kRtLink>(dc, tab, pa, ra);
+        rt_check<kRtLink>(dc, pb, rb);
         rt_store<kRtLink>(dc, pb, rb);
     }
 }
@@ -320,6 +332,7 @@ kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc, const __grid_
     if (!fp8_span(dc, tab, blockIdx.x, sp)) return;              // uniform across the CTA
     RtRegs<kRtHbmVec> r;
     rt_load<kRtHbm>(dc, tab, sp, r);
+    rt_check<kRtHbm>(dc, sp, r);
     rt_store<kRtHbm>(dc, sp, r);
 }
 
