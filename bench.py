@@ -30,7 +30,7 @@ METRIC = "prefix-KV retrieval GB/s and tokens/s on 1 GB300; % of HBM / host-link
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.json")
 # the copy kernels and the async-copy helpers they inline
-KERNEL_SRCS = [os.path.join(ROOT, "paper_2609_35065_gb300", "csrc", f) for f in ("kvs_kernels.cu", "kvs_async.cuh")]
+KERNEL_SRCS = [os.path.join(ROOT, "paper_2609_35065_gb300", "csrc", f) for f in ("kvs_kernels.cu", "kvs_async.cuh", "kvs_job.cuh")]
 HBM_FALLBACK_GBS = 6800.0
 
 
