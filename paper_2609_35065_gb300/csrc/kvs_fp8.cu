@@ -104,9 +104,10 @@ __device__ __forceinline__ bool fp8_piece(const Fp8Job& f, uint32_t q, Fp8Piece&
     return true;
 }
 
-__device__ __forceinline__ uint4 ld_nc16(uint64_t a) {
+// Coherent, not .nc: a programmatic launch exists while the call before it still writes.
+__device__ __forceinline__ uint4 ld_stream16(uint64_t a) {
     uint4 r;
-    asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+    asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(a));
     return r;
 }
@@ -247,8 +248,8 @@ __device__ __forceinline__ void rt_load(const Fp8Spans& dc, const TAB& tab, cons
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint32_t v = threadIdx.x + u * T;
-        if (v < nv) r.c[u] = ld_nc16(sp.codes + (uint64_t)v * 16);
-        r.s[u] = __ldg(reinterpret_cast<const float*>(sp.scales) + fp8_vec_head(dc, sp, min(v, nv - 1)));
+        if (v < nv) r.c[u] = ld_stream16(sp.codes + (uint64_t)v * 16);
+        r.s[u] = reinterpret_cast<const float*>(sp.scales)[fp8_vec_head(dc, sp, min(v, nv - 1))];
         r.blk[u] = tab.block(sp.run0 + fp8_run(dc, sp, min(v, nv - 1) * 16));
     }
 }
@@ -410,7 +411,7 @@ __device__ __forceinline__ void fs_load_regs(const Fp8Job& f, const Fp8Piece& pc
     for (int u = 0; u < kFsVec; ++u) {
         const uint32_t v = threadIdx.x + u * kFsThreads;
         if (v < nv) {
-            r.c[u] = ld_nc16(pc.codes + (uint64_t)v * 16);
+            r.c[u] = ld_stream16(pc.codes + (uint64_t)v * 16);
             r.s[u] = __ldg(reinterpret_cast<const float*>(fs_scale_addr(f, pc, v, h_fixed)));
         }
     }
@@ -591,7 +592,7 @@ __device__ __forceinline__ void store_head_segment(const Fp8Job& f, const TAB& t
             const uint32_t bi = B == 1 ? i : __umulhi(i, f.block_magic), r = i - bi * B;
             const int32_t blk = tab.block(block0 + bi);
             if (blk < 0 || blk >= j.num_blocks) bad = true;
-            else v[u] = ld_nc16(src0 + ((uint64_t)blk * B + r) * row2);
+            else v[u] = ld_stream16(src0 + ((uint64_t)blk * B + r) * row2);
         }
     }
 #pragma unroll
@@ -961,8 +962,8 @@ kvs_fp8_store_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ T
                 if (v < nvec) {
                     const uint64_t src = src_of(v, hh[u]);
                     if (src) {
-                        a[u] = ld_nc16(src);
-                        b[u] = ld_nc16(src + 16);
+                        a[u] = ld_stream16(src);
+                        b[u] = ld_stream16(src + 16);
                         ok[u] = true;
                     } else {
                         bad = true;
@@ -1003,8 +1004,8 @@ kvs_fp8_store_kernel(const __grid_constant__ Fp8Job f, const __grid_constant__ T
                 if (v < nvec) {
                     const uint64_t src = src_of(v, hh[u]);
                     if (src) {
-                        a[u] = ld_nc16(src);
-                        b[u] = ld_nc16(src + 16);
+                        a[u] = ld_stream16(src);
+                        b[u] = ld_stream16(src + 16);
                         ok[u] = true;
                     }
                 }

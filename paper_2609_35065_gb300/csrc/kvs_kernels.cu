@@ -89,15 +89,19 @@ template <> struct Vec<4>  { using T = uint32_t; };
 template <> struct Vec<2>  { using T = uint16_t; };
 template <> struct Vec<1>  { using T = uint8_t; };
 
+// Coherent loads, not .nc ones: those are for data that nothing writes while the kernel
+// exists, and a programmatic launch exists while the call before it, which may write
+// what this one reads, still runs; a load promised to be read-only may be moved above
+// grid_wait().
 template <int V>
 __device__ __forceinline__ typename Vec<V>::T ld_stream(const typename Vec<V>::T* p) {
     if constexpr (V == 16) {
         uint4 r;
-        asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+        asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                      : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
         return r;
     } else {
-        return __ldg(p);
+        return *p;
     }
 }
 
