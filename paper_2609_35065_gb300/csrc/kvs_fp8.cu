@@ -294,10 +294,12 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint
 
 // Host chunks: the next piece's loads are in flight while a piece is converted.  512
 // threads, so that a piece's conversion keeps the next one's loads waiting as little as
-// possible: 24 CTAs hold 207 GB/s alone, where 256 threads x 4 vectors hold 168 and 128
-// x 8 133 to 176.  8192 tokens of the 8B shape on the default grid: 2561 -> 2553 us (the
-// link: 2541).  Beside a GEMM loop 50 to 56 CTAs, two an SM, keep what 100 CTAs of 128
-// threads kept, four an SM: 200 against 201 GB/s with the GEMM at 88% either way.
+// possible: 24 CTAs hold 204 GB/s alone, where 256 threads x 4 vectors hold 168 and 128
+// x 8 133 to 176.  8192 tokens of the 8B shape on the default grid: 2577 -> 2560 us (the
+// link: 2541).  Beside a GEMM loop, 100 CTAs of 128 threads x 8, four an SM, kept 199.5
+// GB/s and 88.4% of the GEMM (86.7 to 89.1% over runs).  56 of these keep 199 and 87.5%,
+// 48 keep 196 and 89%: about 1% less at one of the two, for the gain of capped grids (24
+// CTAs: 165 GB/s and 79.5% of the GEMM -> 183 and 88%).
 template <bool INL>
 __global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
 kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
