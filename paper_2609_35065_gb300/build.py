@@ -3,8 +3,9 @@ binding's marshalling extension beside it.
 
 ``python -m paper_2609_35065_gb300.build`` or ``build_library()``.  Both land in
 ``paper_2609_35065_gb300/_build/`` (git-ignored) and are rebuilt when a source or the
-public header is newer.  The extension needs Python's headers; without them the binding
-marshals with numpy and ctypes only.
+public header is newer.  The extension is optional: where it cannot be built or loaded (no
+Python headers, no C compiler, a folder that cannot be written) the binding marshals with
+numpy and ctypes, after a warning.
 """
 from __future__ import annotations
 
@@ -14,6 +15,7 @@ import shutil
 import subprocess
 import sys
 import sysconfig
+import warnings
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
@@ -68,18 +70,36 @@ def stale(out: str = LIB) -> bool:
 
 
 def pycall_stale() -> bool:
-    return _has_python_headers() and _older(PYCALL, [PYCALL_SOURCE, os.path.join(INCLUDE, "kvs.h")])
+    return _older(PYCALL, [PYCALL_SOURCE, os.path.join(INCLUDE, "kvs.h")])
+
+
+def _usable_pycall(force: bool = False, verbose: bool = False) -> bool:
+    """Whether an extension no older than its sources is there, built now if need be (or forced).
+    One that is older and cannot be rebuilt is not usable: the structs it fills may have changed."""
+    try:
+        if force or pycall_stale():
+            if not _has_python_headers():
+                return False
+            build_pycall(verbose)
+        return True
+    except (OSError, RuntimeError, subprocess.SubprocessError) as e:
+        warnings.warn(f"the binding's extension cannot be built, arguments are marshalled with numpy: {e}",
+                      RuntimeWarning, stacklevel=3)
+        return False
 
 
 def load_pycall():
-    """The extension's ``call``, built first if its source is newer; None without Python's headers."""
-    if pycall_stale():
-        build_pycall()
-    if not os.path.exists(PYCALL):
+    """The extension's ``call``, or None where it cannot be built or loaded."""
+    if not _usable_pycall():
         return None
-    spec = importlib.util.spec_from_file_location("kvs_pycall", PYCALL)
-    mod = importlib.util.module_from_spec(spec)
-    spec.loader.exec_module(mod)
+    try:
+        spec = importlib.util.spec_from_file_location("kvs_pycall", PYCALL)
+        mod = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(mod)
+    except ImportError as e:
+        warnings.warn(f"the binding's extension cannot be loaded, arguments are marshalled with numpy: {e}",
+                      RuntimeWarning, stacklevel=2)
+        return None
     return mod.call
 
 
@@ -95,8 +115,7 @@ def build_pycall(verbose: bool = False) -> None:
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
-    if pycall_stale() or (force and _has_python_headers()):
-        build_pycall(verbose)
+    _usable_pycall(force, verbose)
     if force or stale():
         tmp = LIB + f".{os.getpid()}.tmp"
         cmd = command(tmp)
