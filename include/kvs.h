@@ -359,7 +359,9 @@ int kvs_get_choice(kvs_bw_report* out);
  * KVS_F_FEW_SMS and KVS_F_PREFETCH_L2 flags are KVS_ERR_INVALID_ARG.  When the call holds device-resident chunks, those
  * chunks alone are then timed with the LDG and the TMA kernel (TMA only for
  * 16-byte aligned data), each chunk as a request of its own, and the faster
- * kernel becomes the default for device chunks.  A call with no chunk of a
+ * kernel becomes the default for device chunks.  Calls whose runs (block_size token rows)
+ * are below 16 KiB take that default only if the tuned call's runs were below 16 KiB too;
+ * until then, and again after kvs_query_bw, they take the LDG kernel.  A call with no chunk of a
  * class leaves that class's default unchanged.  `out` (may be NULL) receives
  * the rates in GB/s of each class's bytes (0 for a candidate that cannot
  * serve the call) and the choices.

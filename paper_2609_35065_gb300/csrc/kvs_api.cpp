@@ -112,6 +112,7 @@ struct DevState {
     int          retrieve_host = KVS_VARIANT_HOSTLINK;
     int          store_host = KVS_VARIANT_HOSTLINK;
     int          kernel_device = KVS_KERNEL_LDG;
+    int          kernel_short = KVS_KERNEL_LDG;   // ... for runs below half a piece; kvs_tune of such a call sets it
     size_t       max_pitch = 0;              // largest pitch a 2D copy accepts
     int          hostlink_ctas = 0;          // CTA cap of host-link kernels, 0 = whole GPU
     int          store_ctas = 0;
@@ -445,6 +446,15 @@ int fill_plan(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache,
     // kept writer put into the block.
     if (pl.any_dedup && validate) pl.blocks_cmp = pl.demoted;
     return KVS_OK;
+}
+
+// Runs below half a piece take the LDG kernels' span pieces unless kvs_tune has timed a
+// call of such runs: the TMA kernel moves one run per CTA (16 x 2000 tokens, 24 layers, 4 KiB
+// runs: 127 us in span pieces, 170 us by TMA; 2 KiB: 132 and 273), so what the probe, or a
+// tuned call, found on longer runs says nothing about them.  12 KiB runs are 1.6% faster by
+// TMA (180 and 177 us), which a tuned call finds.
+bool short_runs(const kvs_geometry* g, const Plan& pl) {
+    return (uint64_t)g->block_size * pl.row_bytes < kPieceBytes / 2;
 }
 
 int vec_bytes_for(uint64_t addr_or) {
@@ -785,10 +795,7 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     if (rc) return rc;
     const int grid = (int)KVS_F_GET_MAX_CTAS(flags);
     const int vec = vec_bytes_for(pl.addr_or);
-    // Runs below half a piece take the LDG kernels' span pieces whatever the probe (on
-    // 32 KiB runs) has picked: the TMA kernels move one run per CTA.
-    const bool short_runs = (uint64_t)g->block_size * pl.row_bytes < kPieceBytes / 2;
-    int flavour = f_tma ? KVS_KERNEL_TMA : (f_ldg || short_runs) ? KVS_KERNEL_LDG : st.kernel_device;
+    int flavour = f_tma ? KVS_KERNEL_TMA : f_ldg ? KVS_KERNEL_LDG : short_runs(g, pl) ? st.kernel_short : st.kernel_device;
     if (flavour == KVS_KERNEL_TMA && vec != 16) {
         if (f_tma) return fail(KVS_ERR_UNSUPPORTED, "TMA needs 16-byte aligned chunks, planes and rows");
         flavour = KVS_KERNEL_LDG;
@@ -1251,6 +1258,7 @@ int query_bw(DevState& st, kvs_bw_report* out, cudaStream_t s, int64_t probe_byt
     st.retrieve_host = pick(rep.retrieve_gbs[0], rep.retrieve_gbs[1], rep.retrieve_dma_gbs);
     st.store_host = pick(rep.store_gbs[0], rep.store_gbs[1], rep.store_dma_gbs);
     st.kernel_device = rep.device_kernel_gbs[1] > rep.device_kernel_gbs[0] ? KVS_KERNEL_TMA : KVS_KERNEL_LDG;
+    st.kernel_short = KVS_KERNEL_LDG;
     rep.chosen_retrieve_host = st.retrieve_host;
     rep.chosen_store_host = st.store_host;
     rep.chosen_kernel_device = st.kernel_device;
@@ -1342,6 +1350,7 @@ int tune(DevState& st, const kvs_geometry* g, const kvs_paged_cache* cache, cons
             if (rc) return rc;
         }
         st.kernel_device = rep.device_gbs[1] > rep.device_gbs[0] ? KVS_KERNEL_TMA : KVS_KERNEL_LDG;
+        if (short_runs(g, pl)) st.kernel_short = st.kernel_device;
         rep.chosen_kernel_device = st.kernel_device;
     }
     KVS_CUDA(cudaStreamSynchronize(s));
