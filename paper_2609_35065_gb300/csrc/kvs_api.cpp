@@ -586,8 +586,9 @@ constexpr int kKernelLink = 100;
 constexpr int kKernelLinkPrefetch = 101;   // retrieval only
 constexpr int kKernelLinkStaged = 102;     // retrieval only
 
-int launch_kernel(const Job& j, int flavour, int vec, int grid, cudaStream_t s) {
+int launch_kernel(Job j, int flavour, int vec, int grid, cudaStream_t s) {
     if (j.num_pieces == 0) return KVS_OK;
+    j.early = (flavour == KVS_KERNEL_LDG || flavour == KVS_KERNEL_TMA) && grid == 0;
     cudaError_t e = (flavour == KVS_KERNEL_TMA) ? launch_tma(j, grid, s)
                   : (flavour == kKernelLinkStaged && vec == 16) ? launch_link_staged(j, grid, s)
                   : (flavour == kKernelLinkPrefetch && vec == 16) ? launch_link_prefetch(j, grid, s)
@@ -1066,7 +1067,8 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             if (rc) return rc;
         }
         if (pl.num_device) {
-            const Fp8Job f = fjob(0, pl.num_device, p0, np);
+            Fp8Job f = fjob(0, pl.num_device, p0, np);
+            f.job.early = cap == 0;
             if (f.job.num_pieces >= (1ull << 31) || fp8_segments(f) >= (1ull << 31))
                 return fail(KVS_ERR_INVALID_ARG, "call too large: split it");
             // HBM chunks: uncapped retrievals run one CTA per piece, store-backs stage

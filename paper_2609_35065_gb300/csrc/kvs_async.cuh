@@ -91,8 +91,9 @@ __device__ __forceinline__ void bulk_wait_all() {
 // CTAs scheduled while the stream's previous kernel still runs; grid_wait() then holds
 // them until that kernel has finished and its writes are visible.  grid_trigger():
 // this CTA no longer minds the next such kernel taking up slots.  Only kernels that
-// fill the GPU from HBM trigger, each CTA with its last piece; a host-link kernel runs
-// on a few SMs beside others' work, and its successor's CTAs would hold more of them.
+// fill the GPU from HBM trigger, each CTA with its last piece (Job::early); a host-link
+// kernel, or one under the caller's CTA cap, runs on a few SMs beside others' work, and
+// its successor's CTAs would hold more of them.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

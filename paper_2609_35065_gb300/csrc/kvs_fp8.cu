@@ -904,7 +904,7 @@ kvs_fp8_store_unit_kernel(const __grid_constant__ Fp8Job f, const __grid_constan
             src = source();
         } else {
             mine = 0;
-            if (INL) grid_trigger();
+            if (INL && j.early) grid_trigger();
         }
         const uint64_t inv2 = ((uint64_t)__float_as_uint(inv) << 32) | __float_as_uint(inv);
 #pragma unroll

@@ -62,6 +62,8 @@ struct Job {
     uint32_t        block_size;      // B
     int32_t         mode;            // Mode
     const HostTables* tables;        // not null: entries, blocks and planes are not uploaded
+    uint32_t        early;           // 1: a kernel on HBM chunks without a CTA cap, whose CTAs let the
+                                     // stream's next carried call in (grid_trigger)
     uint32_t        align;           // OR of the plane and chunk addresses and of every n_tok * R (low bits)
 };
 

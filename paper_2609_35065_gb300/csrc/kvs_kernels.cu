@@ -363,7 +363,7 @@ kvs_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ 
     if (INL) grid_wait();
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
-        if (INL && q + gridDim.x >= num_pieces) grid_trigger();
+        if (INL && dc.job.early && q + gridDim.x >= num_pieces) grid_trigger();
         if (!span_piece(dc, tab, q, sp)) continue;            // uniform across the CTA
         if (TAIL && !span_wide(dc, sp)) continue;
         uint4 r[kSpanUnroll];
@@ -382,7 +382,7 @@ kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, const __grid_cons
     if (INL) grid_wait();
     for (uint32_t q = blockIdx.x; q < num_pieces; q += gridDim.x) {
         SpanPiece sp;
-        if (INL && q + gridDim.x >= num_pieces) grid_trigger();
+        if (INL && dc.job.early && q + gridDim.x >= num_pieces) grid_trigger();
         if (!span_piece(dc, tab, q, sp) || span_wide(dc, sp)) continue;   // uniform across the CTA
         const uint32_t a = (uint32_t)sp.chunk | (uint32_t)sp.plane | sp.off | (uint32_t)dc.run_bytes | sp.len;
         if ((a & 7) == 0) span_narrow<MODE, 8, 4>(dc, tab, sp);

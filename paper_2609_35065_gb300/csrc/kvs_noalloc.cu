@@ -330,6 +330,7 @@ int retrieve_noalloc(const kvs_geometry* g, const kvs_paged_cache* cache, const 
     }
     if (ndev) {
         Job jd = j;
+        jd.early = cap == 0;
         jd.entry_base = 0;
         jd.num_entries = (uint32_t)ndev;
         jd.num_pieces = ndev * P * bpc * ppr;

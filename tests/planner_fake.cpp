@@ -12,7 +12,7 @@
 namespace {
 enum Kernel { LDG, TMA, LINK, LINK_STAGED, LINK_PREFETCH, LINK_SIGNAL, FP8_RETRIEVE, FP8_RETRIEVE_STAGED, FP8_STORE, OTHER };
 struct Launch {
-    int kernel, grid, carried;
+    int kernel, grid, carried, early;
 };
 std::vector<Launch> g_seen;
 float g_ms[OTHER + 1];
@@ -20,7 +20,7 @@ int g_last = OTHER;
 
 cudaError_t launched(int kernel, const kvs::Job& j, int grid) {
     g_last = kernel;
-    g_seen.push_back({kernel, grid, j.tables != nullptr});
+    g_seen.push_back({kernel, grid, j.tables != nullptr, (int)j.early});
     return cudaSuccess;
 }
 }  // namespace
@@ -34,7 +34,7 @@ void fake_set_ms(int kernel, float ms) { g_ms[kernel] = ms; }
 int fake_count() { return (int)g_seen.size(); }
 void fake_launch(int k, int* out) {
     const Launch& l = g_seen[k];
-    const int v[] = {l.kernel, l.grid, l.carried};
+    const int v[] = {l.kernel, l.grid, l.carried, l.early};
     for (size_t i = 0; i < sizeof v / sizeof *v; ++i) out[i] = v[i];
 }
 

@@ -54,9 +54,9 @@ class Planner:
         assert getattr(self.lib, name)(*args) == 0, self.lib.kvs_last_error()
         out = []
         for k in range(n, self.lib.fake_count()):
-            v = (ctypes.c_int * 3)()
+            v = (ctypes.c_int * 4)()
             self.lib.fake_launch(k, v)
-            out.append(dict(zip(("kernel", "grid", "carried"), v)))
+            out.append(dict(zip(("kernel", "grid", "carried", "early"), v)))
         return out
 
     def call(self, name, geom, where, tokens=512, flags=0):
@@ -109,3 +109,17 @@ def test_what_was_measured_on_long_runs_does_not_decide_for_short_ones(planner):
     planner._run("kvs_query_bw", None, None, ctypes.c_int64(16 << 20))
     assert _kernels(planner.call("kvs_retrieve", LONG, HBM)) == [TMA]
     assert _kernels(planner.call("kvs_retrieve", SHORT, HBM)) == [LDG]
+
+
+@pytest.mark.parametrize("name", ["kvs_retrieve", "kvs_store", "kvs_retrieve_fp8", "kvs_store_fp8"])
+@pytest.mark.parametrize("geom", [SHORT, LONG, (2, 3, 20, 2, 16, 256)], ids=["4KiB_runs", "32KiB_runs", "120B_rows"])
+def test_only_uncapped_hbm_kernels_let_the_next_call_in_early(planner, geom, name):
+    """The next carried call's CTAs wait on SMs: not beside a copy that the link or the caller's cap bounds."""
+    if "fp8" in name and geom[2] % 16:
+        pytest.skip("fp8 chunks need head_dim a multiple of 16")
+    cap = 4 << 16
+    assert kvs.KVS_F_MAX_CTAS(4) == cap
+    for where, flags, early in ((HBM, 0, 1), (HBM, cap, 0), (HOST, 0, 0), (HOST, cap, 0)):
+        seen = planner.call(name, geom, where, 257, flags)
+        assert [x["early"] for x in seen] == [early], (where, flags, seen)
+        assert all(x["carried"] for x in seen)
