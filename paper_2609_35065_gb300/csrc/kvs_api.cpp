@@ -939,6 +939,10 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     return KVS_OK;
 }
 
+// Two CTAs of the fp8 retrieval share an SM and two SMs a TPC, so four hold a whole TPC; a
+// part of one costs a concurrent GEMM, whose CTA pairs need both SMs, all of it.
+int fp8_link_ctas(int cap) { return cap >= 4 ? cap & ~3 : cap; }
+
 // fp8 chunks (E4M3 codes with per-head binary32 scales) <-> BF16 planes.  Host
 // chunks run first on the host-link grid, device chunks after them on the
 // same stream.  A physical block named by two requests is refused: the
@@ -1053,7 +1057,8 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             const Fp8Job f = fjob(pl.num_device, pl.num_host, p0, np);
             if (f.job.num_pieces >= (1ull << 31) || fp8_segments(f) >= (1ull << 31))
                 return fail(KVS_ERR_INVALID_ARG, "call too large: split it");
-            // Retrieval: an eighth more CTAs than the link kernel (see kvs_fp8_retrieve_kernel).
+            // Retrieval: the link kernel's CTAs, down to a multiple of four (see
+            // kvs_fp8_retrieve_kernel).
             // Store-back: one CTA per (chunk, plane, head) over the whole GPU for a whole call
             // (193 GB/s, the D2H link); layer by layer it runs beside the compute that produces
             // the KV, where a whole-GPU launch per group displaces that compute, so it takes the
@@ -1061,7 +1066,7 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             // 32 CTAs).
             // KVS_F_FEW_SMS: the staged kernel on the BF16 staged kernel's cap (each of its
             // CTAs holds 112 KiB of codes, about what a BF16 staged CTA holds).
-            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? st.hostlink_ctas + st.hostlink_ctas / 8
+            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? fp8_link_ctas(st.hostlink_ctas)
                            : layers_per_step > 0 ? st.store_ctas : 0;
             rc = run(f, grid, false);
             if (rc) return rc;

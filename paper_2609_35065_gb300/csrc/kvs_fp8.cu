@@ -242,14 +242,15 @@ struct RtRegs {
     int32_t blk[U];
 };
 
-template <int T, int U, class TAB>
+// ONE: the vectors of a token row divide T, so that a thread's vectors are all of one head.
+template <int T, bool ONE, int U, class TAB>
 __device__ __forceinline__ void rt_load(const Fp8Spans& dc, const TAB& tab, const Fp8Span& sp, RtRegs<U>& r) {
     const uint32_t nv = sp.len / 16;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const uint32_t v = threadIdx.x + u * T;
         if (v < nv) r.c[u] = ld_stream16(sp.codes + (uint64_t)v * 16);
-        r.s[u] = reinterpret_cast<const float*>(sp.scales)[fp8_vec_head(dc, sp, min(v, nv - 1))];
+        r.s[u] = ONE && u ? r.s[0] : reinterpret_cast<const float*>(sp.scales)[fp8_vec_head(dc, sp, min(v, nv - 1))];
         r.blk[u] = tab.block(sp.run0 + fp8_run(dc, sp, min(v, nv - 1) * 16));
     }
 }
@@ -294,13 +295,13 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint
 
 // Host chunks: the next piece's loads are in flight while a piece is converted.  512
 // threads, so that a piece's conversion keeps the next one's loads waiting as little as
-// possible: 24 CTAs hold 204 GB/s alone, where 256 threads x 4 vectors hold 168 and 128
-// x 8 133 to 176.  8192 tokens of the 8B shape on the default grid: 2577 -> 2560 us (the
-// link: 2541).  Beside a GEMM loop, 100 CTAs of 128 threads x 8, four an SM, kept 199.5
-// GB/s and 88.4% of the GEMM (86.7 to 89.1% over runs).  56 of these keep 199 and 87.5%,
-// 48 keep 196 and 89%: about 1% less at one of the two, for the gain of capped grids (24
-// CTAs: 165 GB/s and 79.5% of the GEMM -> 183 and 88%).
-template <bool INL>
+// possible: 24 CTAs hold 204 GB/s alone, where 256 threads x 4 vectors hold 189 and 128
+// x 8 149.  8192 tokens of the 8B shape take 2564 us on the default grid (the link: 2541).
+// Beside a GEMM loop (averages of 12 runs, all in turn on one GPU) 100 CTAs of 128 threads
+// x 8, four an SM, kept 199.1 GB/s and 87.7% of the GEMM; 56 of these with a scale per
+// vector 198.2 and 86.9%; 48 with one scale a thread (ONE) 197.7 and 88.4%.  50 to 52 of
+// them keep 199 and 87.1%, 56 200 and 86.7%: the step lies at whole TPCs (fp8_link_ctas).
+template <bool ONE, bool INL>
 __global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
 kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
     if (INL) grid_wait();
@@ -308,15 +309,15 @@ kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_consta
     Fp8Span pa, pb;
     uint32_t q = blockIdx.x;
     bool ha = rt_next(dc, tab, q, pa);
-    if (ha) rt_load<kRtLink>(dc, tab, pa, ra);
+    if (ha) rt_load<kRtLink, ONE>(dc, tab, pa, ra);
     while (ha) {
         const bool hb = rt_next(dc, tab, q, pb);
-        if (hb) rt_load<kRtLink>(dc, tab, pb, rb);
+        if (hb) rt_load<kRtLink, ONE>(dc, tab, pb, rb);
         rt_check<kRtLink>(dc, pa, ra);
         rt_store<kRtLink>(dc, pa, ra);
         if (!hb) break;
         ha = rt_next(dc, tab, q, pa);
-        if (ha) rt_load<kRtLink>(dc, tab, pa, ra);
+        if (ha) rt_load<kRtLink, ONE>(dc, tab, pa, ra);
         rt_check<kRtLink>(dc, pb, rb);
         rt_store<kRtLink>(dc, pb, rb);
     }
@@ -334,7 +335,7 @@ kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc, const __grid_
     Fp8Span sp;
     if (!fp8_span(dc, tab, blockIdx.x, sp)) return;              // uniform across the CTA
     RtRegs<kRtHbmVec> r;
-    rt_load<kRtHbm>(dc, tab, sp, r);
+    rt_load<kRtHbm, false>(dc, tab, sp, r);
     rt_check<kRtHbm>(dc, sp, r);
     rt_store<kRtHbm>(dc, sp, r);
 }
@@ -1071,7 +1072,8 @@ cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s) {
     return with_tables(fj.job, [&](const auto& tab) {
         constexpr bool I = std::decay_t<decltype(tab)>::kInline;
         if (per_piece) launch_on(s, tab, kvs_fp8_retrieve_piece_kernel<I>, ctas, kRtHbm, 0, dc, tab);
-        else launch_on(s, tab, kvs_fp8_retrieve_kernel<I>, ctas, kRtLink, 0, dc, tab);
+        else launch_on(s, tab, kRtLink % vpr == 0 ? kvs_fp8_retrieve_kernel<true, I> : kvs_fp8_retrieve_kernel<false, I>,
+                       ctas, kRtLink, 0, dc, tab);
     });
 }
 

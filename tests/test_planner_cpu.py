@@ -123,3 +123,10 @@ def test_only_uncapped_hbm_kernels_let_the_next_call_in_early(planner, geom, nam
         seen = planner.call(name, geom, where, 257, flags)
         assert [x["early"] for x in seen] == [early], (where, flags, seen)
         assert all(x["carried"] for x in seen)
+
+
+def test_fp8_retrieval_from_the_host_holds_whole_tpcs(planner):
+    """Of the 50 CTAs of the built-in cap, 48: four to the two SMs that a GEMM's CTA pair needs."""
+    assert planner.choice().hostlink_ctas == 50
+    assert [x["grid"] for x in planner.call("kvs_retrieve_fp8", LONG, HOST)] == [48]
+    assert [x["grid"] for x in planner.call("kvs_retrieve_fp8", LONG, HOST, flags=kvs.KVS_F_MAX_CTAS(50))] == [50]
