@@ -72,3 +72,20 @@ def test_layer_groups_that_carry_and_that_upload(lps):
         kvs.kvs_retrieve_layers(w.geom, buf.plane_ptrs, w.num_blocks, buf.requests, lps, None, None)
         torch.cuda.synchronize()
         gc.check_retrieve(buf)
+
+
+@pytest.mark.parametrize("flags", [0, kvs.KVS_F_VALIDATE], ids=["carried", "uploaded"])
+@pytest.mark.parametrize("shape", [(3, 8, 128, 16), (2, 2, 64, 16), (2, 5, 256, 16)],
+                         ids=["32KiB_runs", "4KiB_runs", "40KiB_runs"])
+def test_forced_tma_small_calls(shape, flags):
+    """TMA pieces with their tables in the launch's parameters, and uploaded."""
+    L, H, D, B = shape
+    w = synth.custom(L, H, D, B, 256, 80, [600, 256], [512, 256], seed=D, residency="device", store_tokens=[88, 0])
+    buf = buffers.allocate(w, store=True, store_residency="device")
+    assert _table_bytes(w) < 3584
+    args = (w.geom, buf.plane_ptrs, w.num_blocks)
+    kvs.kvs_retrieve(*args, buf.requests, None, kvs.KVS_F_FORCE_TMA | flags)
+    kvs.kvs_store(*args, buf.store_requests, None, kvs.KVS_F_FORCE_TMA | flags)
+    assert kvs.kvs_check_errors(None) == kvs.KVS_OK
+    gc.check_retrieve(buf)
+    gc.check_store(buf)

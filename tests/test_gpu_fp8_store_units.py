@@ -52,3 +52,16 @@ def test_store_units(name, cap, infinities):
                       kvs.KVS_F_VALIDATE | kvs.KVS_F_MAX_CTAS(cap))
     torch.cuda.synchronize()
     gc.check_store_fp8(buf)
+
+
+@pytest.mark.parametrize("name", sorted(SHAPES))
+def test_store_units_with_carried_tables(name):
+    """The ordinary small call: its tables in the launch's parameters (validated calls upload them)."""
+    L, H, D, B, C, tokens = SHAPES[name]
+    nb = sum(-(-t // B) for t in tokens) + 3
+    w = synth.custom(L, H, D, B, C, nb, list(tokens), [0] * len(tokens), seed=D, store_tokens=list(tokens))
+    buf = buffers.allocate_fp8(w, store=True, store_residency="device")
+    _fill(buf, D, True)
+    kvs.kvs_store_fp8(w.geom, buf.plane_ptrs, w.num_blocks, buf.store_requests, None)
+    assert kvs.kvs_check_errors(None) == kvs.KVS_OK
+    gc.check_store_fp8(buf)
