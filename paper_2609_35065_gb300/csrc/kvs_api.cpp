@@ -939,9 +939,17 @@ int copy_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_req
     return KVS_OK;
 }
 
-// Two CTAs of the fp8 retrieval share an SM and two SMs a TPC, so four hold a whole TPC; a
-// part of one costs a concurrent GEMM, whose CTA pairs need both SMs, all of it.
-int fp8_link_ctas(int cap) { return cap >= 4 ? cap & ~3 : cap; }
+// CTAs of an fp8 retrieval of `codes` bytes over the host link, from the link kernel's cap.
+// Two of them share an SM and two SMs a TPC, so four hold a whole TPC; a part of one costs a
+// concurrent GEMM, whose CTA pairs need both SMs, all of it.  One less, because a stride of
+// 48 over the 16 pieces of a full 256-token span gives the pieces that a short last chunk
+// lacks to the same CTAs (chunks of 256 and 44 tokens, 39 MB: 220 us with 48, 194 with 47).
+// Calls of less than 16 MiB are over in 80 us or less and have few pieces a CTA: an eighth
+// more than the cap (1.6 MB 11.5 -> 10.8 us, 4 MB 23.0 -> 22.2; 17 MB 83.4 either way).
+int fp8_link_ctas(int cap, uint64_t codes) {
+    if (codes < (16ull << 20)) return cap + cap / 8;
+    return cap >= 8 ? (cap & ~3) - 1 : cap;
+}
 
 // fp8 chunks (E4M3 codes with per-head binary32 scales) <-> BF16 planes.  Host
 // chunks run first on the host-link grid, device chunks after them on the
@@ -1057,8 +1065,6 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             const Fp8Job f = fjob(pl.num_device, pl.num_host, p0, np);
             if (f.job.num_pieces >= (1ull << 31) || fp8_segments(f) >= (1ull << 31))
                 return fail(KVS_ERR_INVALID_ARG, "call too large: split it");
-            // Retrieval: the link kernel's CTAs, down to a multiple of four (see
-            // kvs_fp8_retrieve_kernel).
             // Store-back: one CTA per (chunk, plane, head) over the whole GPU for a whole call
             // (193 GB/s, the D2H link); layer by layer it runs beside the compute that produces
             // the KV, where a whole-GPU launch per group displaces that compute, so it takes the
@@ -1066,7 +1072,8 @@ int fp8_call(const kvs_geometry* g, const kvs_paged_cache* cache, const kvs_requ
             // 32 CTAs).
             // KVS_F_FEW_SMS: the staged kernel on the BF16 staged kernel's cap (each of its
             // CTAs holds 112 KiB of codes, about what a BF16 staged CTA holds).
-            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? fp8_link_ctas(st.hostlink_ctas)
+            const uint64_t codes = f.tokens * np * hd;
+            const int grid = cap ? cap : few ? st.few_sm_ctas : retrieve ? fp8_link_ctas(st.hostlink_ctas, codes)
                            : layers_per_step > 0 ? st.store_ctas : 0;
             rc = run(f, grid, false);
             if (rc) return rc;

@@ -297,10 +297,10 @@ __device__ __forceinline__ bool rt_next(const Fp8Spans& dc, const TAB& tab, uint
 // threads, so that a piece's conversion keeps the next one's loads waiting as little as
 // possible: 24 CTAs hold 204 GB/s alone, where 256 threads x 4 vectors hold 189 and 128
 // x 8 149.  8192 tokens of the 8B shape take 2564 us on the default grid (the link: 2541).
-// Beside a GEMM loop (averages of 12 runs, all in turn on one GPU) 100 CTAs of 128 threads
-// x 8, four an SM, kept 199.1 GB/s and 87.7% of the GEMM; 56 of these with a scale per
-// vector 198.2 and 86.9%; 48 with one scale a thread (ONE) 197.7 and 88.4%.  50 to 52 of
-// them keep 199 and 87.1%, 56 200 and 86.7%: the step lies at whole TPCs (fp8_link_ctas).
+// Beside a GEMM loop (averages of 8 to 12 runs, in turn on one GPU) 100 CTAs of 128 threads
+// x 8, four an SM, kept 199 GB/s and 87.7% of the GEMM; 56 of these with a scale per vector
+// 198 and 86.8%; 47 or 48 with one scale a thread (ONE) 197.5 and 88.2%.  49 to 52 of them
+// keep 199 and 87.0%, 56 200 and 86.7%: the step lies at whole TPCs (fp8_link_ctas).
 template <bool ONE, bool INL>
 __global__ void __launch_bounds__(kRtLink, kRtLinkCtas)
 kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
@@ -324,7 +324,9 @@ kvs_fp8_retrieve_kernel(const __grid_constant__ Fp8Spans dc, const __grid_consta
 }
 
 // HBM chunks: one CTA per piece, no persistence; six CTAs per SM (four, or 128 threads x 8
-// vectors, or 512 x 2: up to 1% slower).
+// vectors, or 512 x 2: up to 1% slower).  With carried tables the 40 registers spill 16
+// bytes; five CTAs do not (8 x 2048 tokens 470.3 -> 471.1 us, one 256-token chunk 12.6 ->
+// 11.5).
 template <bool INL>
 __global__ void __launch_bounds__(kRtHbm, kRtHbmCtas)
 kvs_fp8_retrieve_piece_kernel(const __grid_constant__ Fp8Spans dc, const __grid_constant__ Tables<INL> tab) {
@@ -369,7 +371,7 @@ __device__ __forceinline__ bool rt_next(const Fp8Job& f, uint32_t n, uint32_t& q
 // thread copies, with cp.async, its own 16-code vectors and the binary32 scale
 // of each vector's head into slots that only it reads back (no CTA barrier).
 // 100 KiB of shared memory per CTA, two CTAs per SM: 224 KiB of codes in flight
-// per SM, where kvs_fp8_retrieve_kernel holds 128 KiB.  Piece i of a CTA lives
+// per SM, where kvs_fp8_retrieve_kernel holds 64 KiB.  Piece i of a CTA lives
 // in slot i % 7; pieces come in grid-stride order, so once a slot finds none
 // left, neither does any slot after it.
 constexpr int kFsThreads = 256;
@@ -1068,12 +1070,13 @@ cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s) {
     uint32_t piece = kFp8PieceCodes;
     while (piece > kFp8PieceCodes / 4 && total / piece < 2ull * (per_piece ? sm_count() : grid)) piece /= 2;
     const Fp8Spans dc = make_spans(fj, piece);
+    // One scale a thread gains beside other work only, and costs the smallest calls 0.1 us.
+    const bool one = kRtLink % vpr == 0 && piece == kFp8PieceCodes;
     const uint32_t ctas = per_piece ? dc.num_pieces : std::min<uint32_t>((uint32_t)grid, dc.num_pieces);
     return with_tables(fj.job, [&](const auto& tab) {
         constexpr bool I = std::decay_t<decltype(tab)>::kInline;
         if (per_piece) launch_on(s, tab, kvs_fp8_retrieve_piece_kernel<I>, ctas, kRtHbm, 0, dc, tab);
-        else launch_on(s, tab, kRtLink % vpr == 0 ? kvs_fp8_retrieve_kernel<true, I> : kvs_fp8_retrieve_kernel<false, I>,
-                       ctas, kRtLink, 0, dc, tab);
+        else launch_on(s, tab, one ? kvs_fp8_retrieve_kernel<true, I> : kvs_fp8_retrieve_kernel<false, I>, ctas, kRtLink, 0, dc, tab);
     });
 }
 

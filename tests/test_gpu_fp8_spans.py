@@ -23,6 +23,8 @@ SHAPES = {
     "head_176_rows_cross_pieces": (2, 5, 176, 3, 48, (200, 47)),
     "one_vector": (1, 1, 16, 1, 1, (1,)),
     "all_chunks_short": (3, 2, 64, 16, 256, (42, 17, 33)),
+    "rows_of_512_vectors": (1, 64, 128, 4, 64, (130, 3)),    # a thread's vectors are still of one head
+    "rows_of_1024_vectors": (1, 128, 128, 2, 32, (73,)),
 }
 
 

@@ -126,7 +126,11 @@ def test_only_uncapped_hbm_kernels_let_the_next_call_in_early(planner, geom, nam
 
 
 def test_fp8_retrieval_from_the_host_holds_whole_tpcs(planner):
-    """Of the 50 CTAs of the built-in cap, 48: four to the two SMs that a GEMM's CTA pair needs."""
+    """Of the 50 CTAs of the built-in cap, 47, on the SMs of 48: four CTAs to the two SMs that a
+    GEMM's CTA pair needs, and no common factor with a span's pieces.  Calls of less than 16 MiB
+    of codes take an eighth more than the cap."""
     assert planner.choice().hostlink_ctas == 50
-    assert [x["grid"] for x in planner.call("kvs_retrieve_fp8", LONG, HOST)] == [48]
-    assert [x["grid"] for x in planner.call("kvs_retrieve_fp8", LONG, HOST, flags=kvs.KVS_F_MAX_CTAS(50))] == [50]
+    grid = lambda geom, tokens, flags=0: planner.call("kvs_retrieve_fp8", geom, HOST, tokens, flags)[0]["grid"]
+    assert grid((32, 8, 128, 2, 16, 256), 256) == grid((32, 8, 128, 2, 16, 256), 2000) == 47
+    assert grid(LONG, 512) == grid((32, 8, 128, 2, 16, 256), 255) == 56
+    assert grid(LONG, 512, kvs.KVS_F_MAX_CTAS(50)) == 50
