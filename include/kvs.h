@@ -196,7 +196,7 @@ int kvs_store(const kvs_geometry* geom, const kvs_paged_cache* cache,
  * Layer-wise retrieval.  The paper's time-to-use ends when retrieval begins,
  * not when the model consumes the KV (Sec. 3.1): the model can start on the
  * first layers while later layers are still in flight.  This call does the
- * same copy as kvs_retrieve, planned and uploaded once, as ceil(L /
+ * same copy as kvs_retrieve, planned once, as ceil(L /
  * layers_per_step) launch groups in layer order on cuda_stream; after group k
  * (layers [k * layers_per_step, (k + 1) * layers_per_step)) is enqueued,
  * layer_events[k] is recorded on cuda_stream, so another stream can
@@ -442,10 +442,12 @@ int64_t kvs_stat_launches(void);
  *    (once per device, with that device current); make that first call
  *    before any stream capture.  kvs_shutdown() forgets the address, so
  *    after a cudaDeviceReset call kvs_shutdown() before the next call;
- *  - every call shares the one array and overwrites it: calls whose work can
+ *  - every call may use and overwrite the one array: calls whose work can
  *    overlap on the GPU (different streams, or other host threads) race and
- *    must be ordered by the caller; calls in order on one stream are safe;
- *    the error word is cleared at the start of each call;
+ *    must be ordered by the caller; calls in order on one stream are safe.
+ *    (A small unvalidated call passes its tables with the launch and leaves
+ *    the array alone.)  The error word is cleared at the start of each call
+ *    that writes its tables there, validated calls among them;
  *  - every chunk pointer is checked as kvs_retrieve's KVS_F_VALIDATE checks
  *    it (mapped page-locked host memory, or device memory), on every call;
  *  - host chunks are always read directly over the host link, by the same

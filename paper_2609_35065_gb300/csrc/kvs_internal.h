@@ -119,9 +119,10 @@ struct Fp8Job {
     uint32_t ragged;             // 1 when some entry holds fewer tokens than another
 };
 constexpr uint32_t kFp8MaxHeads = 128;
-// Retrieval: a persistent grid of `grid` CTAs (<= 0: fill the GPU) over pieces of at
+// Retrieval: a persistent grid of `grid` CTAs (0: fill the GPU) over span pieces of at
 // most 16 KiB of codes, double-buffered; grid == kFp8PerPiece: one CTA per piece
-// (HBM sources).  The number of pieces is in job.num_pieces.
+// (HBM sources).  job.num_pieces counts pieces of single runs, which the staged kernel
+// walks; the span pieces are cut at the launch.
 constexpr int kFp8PerPiece = -1;
 cudaError_t launch_fp8_retrieve(const Fp8Job& fj, int grid, cudaStream_t s);
 // Retrieval of host chunks with more codes in flight per SM (two pieces in

@@ -6,7 +6,7 @@
 // (layer, K/V) plane [NB][B][H][D].  Two flavours:
 //
 //  * LDG: the threads of a CTA move one 32 KiB piece with 16-byte vector
-//    loads (non-coherent, no L1 allocation) issued ahead of 16-byte streaming
+//    loads (coherent, no L1 allocation) issued ahead of 16-byte streaming
 //    stores.  Uncapped 16-byte work runs one 512-thread, 28-register CTA per
 //    piece (kvs_ldg_piece_kernel, four CTAs per SM).  Runs below half a piece,
 //    capped grids and odd alignments run over span pieces, 32 KiB of the
@@ -352,7 +352,8 @@ __device__ __forceinline__ void span_narrow(const SpanDecoder& dc, const TAB& ta
 // TAIL some pieces are not wide, or end in a tail.  512 threads x 4 vectors on 32
 // registers: four CTAs and 128 KiB of loads in flight per SM.  Three CTAs (40
 // registers) lose nothing on retrievals but 16% on store-backs, whose loads wait
-// for their lookups (4 KiB runs: 139 us against 119).
+// for their lookups (4 KiB runs: 139 us against 119).  With uploaded tables the 32
+// registers spill 8 bytes (store) or 16 (retrieval).
 constexpr int kSpanThreads = 512;
 constexpr int kSpanCtasPerSm = 4;
 constexpr int kSpanUnroll = kPieceBytes / 16 / kSpanThreads;
@@ -375,7 +376,11 @@ kvs_span_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ 
 }
 
 // The other pieces, in a kernel of its own: as a branch of the one above, its
-// registers spill there or halve its CTAs (aligned 120-byte rows: 9.4 -> 13 us).
+// registers spill there or halve its CTAs (aligned 120-byte rows: 9.4 -> 13 us).  Here
+// they spill too, 68 to 144 bytes at the 40 registers of three CTAs an SM.  Two CTAs do
+// not spill and are slower from HBM where runs are copied one by one (B = 1, rows of 4662
+// bytes: 99 -> 132 us; 120-byte runs 1 to 5%), but faster for short runs over the link
+// (120-byte runs, 47 MB: 291 -> 262 us retrieved, 317 -> 305 stored).
 template <int MODE, bool INL>
 __global__ void __launch_bounds__(kSpanThreads, 3)
 kvs_span_narrow_kernel(const __grid_constant__ SpanDecoder dc, const __grid_constant__ Tables<INL> tab, uint32_t num_pieces) {
@@ -909,10 +914,6 @@ int clamp_grid(int grid, int per_sm, uint64_t pieces) {
     return grid < 1 ? 1 : grid;
 }
 
-// With no cap, one CTA per piece: the hardware block scheduler keeps every SM
-// busy and overlaps one CTA's stores with the next CTA's loads.  Measured on a
-// 2 GiB HBM copy this reaches 7.1 TB/s (read + write) against 6.5-6.7 TB/s for
-// persistent grid-stride grids of any shape.
 SpanDecoder make_span_decoder(const Job& job, uint32_t piece_bytes) {
     SpanDecoder dc;
     dc.job = job;
@@ -1058,6 +1059,11 @@ int tma_ctas_per_sm() { return 1; }
 // per piece of a run.  Shorter runs, capped grids and odd alignments: span pieces.
 // 12 KiB runs take 173 us as span pieces and 179 as runs (172 by TMA), 16 KiB
 // runs 226.5 us either way, and 20 KiB runs 281.8 us either way.
+//
+// With no cap, one CTA per piece: the hardware block scheduler keeps every SM
+// busy and overlaps one CTA's stores with the next CTA's loads.  Measured on a
+// 2 GiB HBM copy this reaches 7.1 TB/s (read + write) against 6.5-6.7 TB/s for
+// persistent grid-stride grids of any shape.
 cudaError_t launch_ldg(const Job& job, int vec_bytes, int grid, cudaStream_t s) {
     if (job.num_pieces == 0) return cudaSuccess;
     if (job.mode == MODE_COMPARE) return launch_compare(job, vec_bytes, grid, s);
