@@ -44,6 +44,8 @@ CASES = {
     "fp8_wide_units": (True, 6, 80, 16, 256, (512, 300), 0),
     "fp8_clusters": (True, 3, 256, 16, 256, (512, 300), 0),
     "fp8_capped": (True, 8, 128, 16, 256, (256, 200), kvs.KVS_F_MAX_CTAS(7)),
+    "fp8_clusters_capped": (True, 3, 256, 16, 256, (256, 200), kvs.KVS_F_MAX_CTAS(9)),
+    "fp8_wide_units_capped": (True, 6, 80, 16, 256, (256, 200), kvs.KVS_F_MAX_CTAS(9)),
 }
 
 
